@@ -2,6 +2,7 @@
 // previous kernel's tail, and the register-tiled convolution both directions use.
 #pragma once
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 
@@ -78,6 +79,73 @@ inline bool smem_limit(Kernel kernel, int bytes, bool (&done)[64]) {
         done[dev] = true;
     }
     return true;
+}
+
+// A kernel launched as clusters of up to 16 CTAs: its per-device attributes, and how many clusters of each size a device runs at
+// the same time (a cluster lies within one group of SMs).
+struct ClusterKernel {
+    bool smem[64] = {}, wide[64] = {};
+    std::atomic<int> resident[64][17] = {};
+};
+template <typename Kernel>
+inline bool cluster_attributes(ClusterKernel& k, Kernel kernel, int max_smem) {
+    int dev = -1;
+    if (!smem_limit(kernel, max_smem, k.smem) || cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (!k.wide[dev]) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+        k.wide[dev] = true;
+    }
+    return true;
+}
+inline cudaLaunchAttribute cluster_of(int ctas) {
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = ctas;
+    a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    return a;
+}
+// (0 where it cannot be told)
+template <typename Kernel>
+inline int resident_clusters(ClusterKernel& k, Kernel kernel, int max_smem, int ctas, int threads) {
+    int dev = -1;
+    if (!cluster_attributes(k, kernel, max_smem) || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    int n = k.resident[dev][ctas].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = max_smem;
+        cudaLaunchAttribute attr = cluster_of(ctas);
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        k.resident[dev][ctas].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+template <typename... Params, typename... Args>
+inline bool launch_clusters(ClusterKernel& k, void (*kernel)(Params...), int max_smem, int ctas, int clusters, int threads, size_t smem, cudaStream_t st, const Args&... args) {
+    if (!cluster_attributes(k, kernel, max_smem)) return false;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(clusters * ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1] = cluster_of(ctas);
+    cfg.attrs = attr;
+    cfg.numAttrs = ctas > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
 }
 
 // Two fp32 FMAs per instruction (each rounded as an FMA of its own): the kernels here are bound by instruction issue, and a

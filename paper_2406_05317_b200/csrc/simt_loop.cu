@@ -1,20 +1,22 @@
-// Algorithm 2's whole chunk loop in one launch, for small fp32 problems: a block of 512 threads owns one (sequence, head)
-// unit and keeps its cache, its conv weights and the chunk at hand in shared memory.
+// Algorithm 2's whole chunk loop in one launch, for small fp32 problems: a cluster of 1 to 16 CTAs of 512 threads owns one
+// (sequence, head) unit; every CTA keeps the unit's whole [cache; chunk] in shared memory.
 //
 // Such a problem is all latency: with M = B = 16, d = 64, k = 5 a chunk is 280 thousand FMAs, a microsecond of one SM,
 // and through the per-chunk launches (three per chunk, 2 to 3 us each on the host alone) 256 tokens took 252 us.
-// Here a chunk is three phases between block barriers:
-//   1. scores Q K^T by some of the warps, beside the convolution of Eq. 6 with bias and ReLU by the others
-//   2. maximum and exponentials of every query's scores
-//   3. O = P V / sum P, and the new cache = R [X_K | X_V] / (sum R + eps) into the other of two cache buffers
-// while the next chunk's rows are on their way (asynchronous copies into the other chunk buffer).
-// Bound: shared-memory reads and the latencies of the three phases. The products of phase 1 are tiles (4 x 4 scores, 4 slots
-// x 8 positions of the convolution) whose channels are spread over the lanes of a group, four each, so that even 16 x 32
-// results occupy many warps; the lanes' sums meet in shuffles. In phase 3 a thread owns whole results (a few rows x four
-// channels) and reads every position: no sums to exchange, and the row sums fall out on the way. (With both spread over
-// eight lanes per result the phase took 2.4 us of a chunk's 6.3 at M = B = 16, d = 64; the convolution in 4 x 4 tiles by
-// all warps, after the scores, 2.1.)
+// The CTAs of a cluster share the slots and the chunk's queries: a CTA convolves for its own slots over all positions, so that
+// their rows of R, their denominators and their new cache rows are its own affair, and it writes those rows into the shared
+// memory of all CTAs; one cluster barrier per chunk is all the exchange there is. Within a CTA two groups of warps work side by side:
+//   the chain   convolution of Eq. 6 with bias and ReLU -> barrier of these warps -> new rows R [X_K | X_V] / (sum R + eps), into the
+//               other of two row buffers, of every CTA
+//   attention   a warp takes up to four queries from scores to output, with no barrier at all; before that these warps ask for the
+//               next chunk's rows (asynchronous copies into the other buffer)
+// The convolution is tiles of 2 to 4 slots x 4 or 8 positions whose channels are spread over the lanes of a group, so that few
+// results occupy many warps; the lanes' sums meet in shuffles. Positions of a blend are spread over up to eight lanes likewise.
+// Bound: the latencies of the chain (dependent loads and FMAs at about 3 cycles per instruction, 12 warps or 24 alike).
+// us per call, a block per unit with four rounds of block barriers -> now: 256 tokens, M = B = 16, d = 64, k = 5 76 -> 41 (8 CTAs per unit;
+// of 4 47, of 2 56, one 66; 148 units, one each 81 -> 69); 777 tokens of 8 units, M = 48, B = 100 180 (launches) -> 72 (10 CTAs).
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -26,8 +28,9 @@ namespace {
 
 using namespace simt;
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 512, kWarps = kThreads / 32;
 constexpr int kMaxSmem = 232448 - 128;   // dynamic shared memory: 227 KB less the kernel's few static words
+constexpr int kMaxCluster = 16;
 
 struct LoopParams {
     View q, k, v, o, k_cache, v_cache;
@@ -37,13 +40,15 @@ struct LoopParams {
     float eps, scale;
     float *snap_k, *snap_v;      // optional: [chunk][units][M][d]
     int64_t snap_step;           // floats between chunks
-    int conv_warps;              // warps 0 .. conv_warps - 1 compute the convolution, the others the scores
     float* lse;                  // optional: [units][L]
+    int ctas;                    // CTAs per unit
+    int chain_warps;             // warps 0 .. chain_warps - 1 update the cache, the others (an even number) attend
+    int tile;                    // slots x positions of a convolution tile: 0, 1, 2: 4, 3, 2 x 8; 3: 2 x 4
 };
 
 __host__ __device__ inline int round4(int x) { return (x + 3) / 4 * 4; }
 // Shared memory, in floats. A buffer of rows holds [zeros | cache | chunk | zeros], keys and values side by side, so that a
-// row of [cache; chunk] and the convolution's padding are plain offsets; while a compress step reads one buffer it writes
+// row of [cache; chunk] and the convolution's padding are plain offsets; while a compress step reads one buffer the CTAs write
 // the new cache into the other, where the next chunk is on its way. Row strides are padded by four so that lanes that take
 // consecutive rows meet different banks.
 template <int D>
@@ -51,22 +56,23 @@ struct Strides {
     static constexpr int kRow = 2 * D + 4, kQuery = D + 4;
 };
 struct LoopLayout {
-    int PS, MS;                  // row strides of P^T (queries along the row) and R^T (slots along the row)
+    int MS;                      // row stride of R^T (this CTA's slots along the row)
     int rows;                    // per buffer
-    int g, x, q, p, r, top, total;
+    int queries;                 // per buffer
+    int g, x, q, p, r, total;
 };
-__host__ __device__ inline LoopLayout loop_layout(int d, int M, int B, int k, int c_in) {
+__host__ __device__ inline LoopLayout loop_layout(int d, int M, int B, int k, int c_in, int ctas, int attention_warps) {
     LoopLayout l;
-    l.PS = round4(B) + 4;
-    l.MS = round4(M) + 4;
+    const int slots = round4((M + ctas - 1) / ctas);
+    l.MS = slots + 4;
     l.rows = M + B + k - 1 + 8;
+    l.queries = (B + ctas - 1) / ctas;
     int off = 0;
-    l.g = off;      off += round4(M) * k * c_in;
+    l.g = off;      off += slots * k * c_in;
     l.x = off;      off += 2 * l.rows * (2 * d + 4);
-    l.q = off;      off += 2 * (B + 3) * (d + 4);
-    l.p = off;      off += (M + B + 3) * l.PS;
+    l.q = off;      off += 2 * l.queries * (d + 4);
+    l.p = off;      off += attention_warps * (M + B) * 4;  // [warp][key][up to four queries]
     l.r = off;      off += (M + B + 7) * l.MS;
-    l.top = off;    off += round4(B);
     l.total = off;
     return l;
 }
@@ -93,50 +99,88 @@ __device__ __forceinline__ void reduce_lanes(float (&v)[N], int lane) {
     }
 }
 
-// One row of a tile of dot products: acc[b] += over this lane's four channels x . y[b]
+// One row of a tile of dot products: acc[b] += over this lane's four channels x . y[(b + first) % NB]
 template <int NB>
-__device__ __forceinline__ void row_fma(const f32x4& x, const f32x4 (&y)[NB], f32x2* acc) {
+__device__ __forceinline__ void row_fma(const f32x4& x, const f32x4 (&y)[NB], int first, f32x2* acc) {
 #pragma unroll
-    for (int b = 0; b < NB; ++b) { fma2(x.lo, y[b].lo, acc[b]); fma2(x.hi, y[b].hi, acc[b]); }
+    for (int b = 0; b < NB; ++b) { fma2(x.lo, y[(b + first) % NB].lo, acc[b]); fma2(x.hi, y[(b + first) % NB].hi, acc[b]); }
 }
 
-// kLC: lanes that share a convolution tile's channels (c_in / 4, at most 32)
+// N floats at dst, in all CTAs of the cluster
+template <int N>
+__device__ __forceinline__ void store_everywhere(float* dst, const float* v, int rank, int ctas) {
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(dst);
+#pragma unroll 4
+    for (int c = 0; c < ctas; ++c) {
+        const uint32_t r = remote(at, rank + c < ctas ? rank + c : rank + c - ctas);
+        if constexpr (N == 4) asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(r), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+        else if constexpr (N == 2) asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(r), "f"(v[0]), "f"(v[1]) : "memory");
+        else st_remote(r, v[0]);
+    }
+}
+
+// N floats at an address that is a multiple of their size
+template <int N>
+__device__ __forceinline__ void get(const float* src, float (&v)[N]) {
+    if constexpr (N == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(src);
+    else if constexpr (N == 2) *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(src);
+    else v[0] = src[0];
+}
+template <int N>
+__device__ __forceinline__ void put(float* dst, const float (&v)[N]) {
+    if constexpr (N == 4) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(v);
+    else if constexpr (N == 2) *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(v);
+    else dst[0] = v[0];
+}
+
+// kLC: lanes that share a small convolution tile's channels (c_in / 4, at most 32); half as many share a large one's
 template <int D, int kLC>
 __global__ void __launch_bounds__(kThreads, 1) small_loop_kernel(const __grid_constant__ LoopParams P) {
     extern __shared__ __align__(16) float smem[];
     constexpr int kLD = D / 4, RS = Strides<D>::kRow, RQ = Strides<D>::kQuery;
-    __shared__ const float* src_base[3];
-    __shared__ int64_t src_stride[3];
-    const int u = blockIdx.x, n = u / P.heads, h = u % P.heads;
+    const int ctas = P.ctas, rank = blockIdx.x % ctas, u = blockIdx.x / ctas, n = u / P.heads, h = u % P.heads;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int M = P.M, B = P.B, k = P.k_taps, C = P.c_in, pad = (k - 1) / 2;
-    const LoopLayout lay = loop_layout(D, M, B, k, C);
-    const int PS = lay.PS, MS = lay.MS;
-    float *Gs = smem + lay.g, *Ps = smem + lay.p, *Rs = smem + lay.r, *top = smem + lay.top;
+    const int i_begin = M * rank / ctas, slots = M * (rank + 1) / ctas - i_begin;      // this CTA's slots
+    const int chain_warps = P.chain_warps, chain_threads = 32 * chain_warps;
+    const LoopLayout lay = loop_layout(D, M, B, k, C, ctas, kWarps - chain_warps);
+    const int MS = lay.MS;
+    float *Gs = smem + lay.g, *Ps = smem + lay.p + (warp - chain_warps) * (M + B) * 4, *Rs = smem + lay.r;
     auto rows_of = [&](int buf) { return smem + lay.x + (buf * lay.rows + pad) * RS; };      // row 0 of [cache; chunk]
-    start_and_wait();
-    if (tid < 3) {
-        const View& v = tid == 0 ? P.k : (tid == 1 ? P.v : P.q);
-        src_base[tid] = unit_base<float>(v, n, h);
-        src_stride[tid] = v.st;
-    }
-    for (int x = tid; x < 2 * lay.rows * RS; x += kThreads) smem[lay.x + x] = 0.f;
+    auto everybody = [&] {
+        if (ctas == 1) __syncthreads();
+        else cluster_sync();
+    };
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int x = tid; x < 2 * lay.rows * RS / 4; x += kThreads) store4(smem + lay.x + 4 * x, make_float4(0.f, 0.f, 0.f, 0.f));
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
 
-    // the chunk's keys and values into rows c .. of row buffer `buf`, its queries into query buffer `qbuf`
+    // The attention's threads bring the chunk's keys and values into rows c .. of row buffer `buf` (zeros behind a short one), and this
+    // CTA's queries (every ctas-th, so that all CTAs have early and late ones) into query buffer `qbuf`. A thread copies the
+    // same four channels of every step-th row.
+    const int at = tid - chain_threads, step = (kThreads - chain_threads) / (2 * kLD);
+    const int row0 = at / (2 * kLD), ch0 = 4 * (at % (2 * kLD)), q_row0 = at / kLD, q_ch0 = 4 * (at % kLD);
+    const View& kv = ch0 < D ? P.k : P.v;
+    const float* kv_src = unit_base<float>(kv, n, h) + row0 * kv.st + (ch0 < D ? ch0 : ch0 - D);
+    const float* q_src = unit_base<float>(P.q, n, h) + (rank + q_row0 * ctas) * P.q.st + q_ch0;
+    const int64_t kv_step = step * kv.st, q_step = (int64_t)2 * step * ctas * P.q.st;
     auto fetch = [&](int t0, int c, int buf, int qbuf) {
         const int b = min(B, P.L - t0);
-        float *rows = rows_of(buf) + c * RS, *qs = smem + lay.q + qbuf * (B + 3) * RQ;
-        for (int x = tid; x < b * 3 * kLD; x += kThreads) {
-            const int r = x / (3 * kLD), q4 = x % (3 * kLD), which = q4 / kLD, ch = 4 * (q4 % kLD);
-            cp_async16(which == 2 ? qs + r * RQ + ch : rows + r * RS + which * D + ch, src_base[which] + (t0 + r) * src_stride[which] + ch, true);
-        }
+        float *rows = rows_of(buf) + c * RS, *dst = rows + row0 * RS + ch0;
+        const float* src = kv_src + t0 * kv.st;
+        for (int r = row0; r < b; r += step, dst += step * RS, src += kv_step) cp_async16(dst, src, true);
+        dst = smem + lay.q + (qbuf * lay.queries + q_row0) * RQ + q_ch0;
+        src = q_src + t0 * P.q.st;
+        for (int q = rank + q_row0 * ctas; q < b; q += 2 * step * ctas, dst += 2 * step * RQ, src += q_step) cp_async16(dst, src, true);
         cp_async_commit();
+        if (c + b < M + B)
+            for (int x = at; x < pad * RS / 4; x += kThreads - chain_threads) store4(rows + b * RS + 4 * x, make_float4(0.f, 0.f, 0.f, 0.f));
     };
-    fetch(0, P.c0, 0, 0);
+    if (at >= 0) fetch(0, P.c0, 0, 0);
     {
-        const float* g = P.g_reverse + (P.weights_per_head ? (int64_t)h * M * k * C : 0);
-        const int live = M * k * C / 4, all = round4(M) * k * C / 4;
+        const float* g = P.g_reverse + ((int64_t)(P.weights_per_head ? h * M : 0) + i_begin) * k * C;
+        const int live = slots * k * C / 4, all = (MS - 4) * k * C / 4;
         for (int x = tid; x < all; x += kThreads) cp_async16(Gs + 4 * x, x < live ? g + 4 * x : g, x < live);
         for (int x = tid; x < P.c0 * 2 * kLD; x += kThreads) {
             const int r = x / (2 * kLD), q4 = x % (2 * kLD), c = 4 * (q4 % kLD);
@@ -145,161 +189,234 @@ __global__ void __launch_bounds__(kThreads, 1) small_loop_kernel(const __grid_co
         }
         cp_async_commit();
     }
+    const int full_queries = (B - rank + ctas - 1) / ctas, tail_queries = ((P.L - 1) % B + ctas - rank) / ctas;
     const float sc2 = P.scale * 1.4426950408889634f;
     const int n_chunks = (P.L + B - 1) / B;
     int c = P.c0, cur = 0;
+    cp_async_wait<0>();
+    everybody();
 #pragma unroll 1
     for (int ch = 0; ch < n_chunks; ++ch) {
+        // (this chunk is there, and nobody, here or in another CTA, reads the other buffers any more)
         const int t0 = ch * B, b = min(B, P.L - t0), S = c + b;
         const bool compress = S > M;
         float* X = rows_of(cur);
-        const float* qs = smem + lay.q + (ch & 1) * (B + 3) * RQ;
-        cp_async_wait<0>();
-        if (compress && S < M + B)                          // a short chunk, or the first to be compressed: zeros behind it
-            for (int x = tid; x < pad * RS; x += kThreads) X[S * RS + x] = 0.f;
-        __syncthreads();                                    // this chunk is there, and nobody reads the other buffers any more
-        if (ch + 1 < n_chunks) fetch(t0 + B, compress ? M : S, compress ? cur ^ 1 : cur, (ch + 1) & 1);
-        if (P.snap_k) {
-            for (int x = tid; x < c * 2 * kLD; x += kThreads) {
-                const int r = x / (2 * kLD), q4 = x % (2 * kLD);
-                float* dst = (q4 < kLD ? P.snap_k : P.snap_v) + ch * P.snap_step + ((int64_t)u * M + r) * D + 4 * (q4 % kLD);
-                store4(dst, load4(X + r * RS + 4 * q4));
+        if (at >= 0) {
+            if (ch + 1 < n_chunks) fetch(t0 + B, compress ? M : S, compress ? cur ^ 1 : cur, (ch + 1) & 1);
+            if (P.snap_k) {
+                float* snap = (ch0 < D ? P.snap_k : P.snap_v - D) + ch * P.snap_step + (int64_t)u * M * D + ch0;
+                for (int r = rank * step + row0; r < c; r += ctas * step) store4(snap + r * D, load4(X + r * RS + ch0));
             }
-        }
-        const int conv_warps = compress ? P.conv_warps : 0;
-        if (warp >= conv_warps) {
-            // ---- 1a. scores, P^T[key][query], in base-2 units; masked entries -inf
-            constexpr int kLanes = D / 8, kPerWarp = 32 / kLanes, kOut = 16 / kLanes;      // eight channels per lane
-            const int qt = (b + 3) / 4, kt = (S + 3) / 4, tiles = qt * kt, gl = tid % kLanes;
+            // ---- attention: scores (in base-2 units, masked entries -inf), maximum, exponentials, O = P V / sum P
+            const int queries = b == B ? full_queries : tail_queries;
+            const float* qs = smem + lay.q + (ch & 1) * lay.queries * RQ;
+            auto attend = [&](auto per_warp) {
+                constexpr int Q = decltype(per_warp)::value;
 #pragma unroll 1
-            for (int t0w = (warp - conv_warps) * kPerWarp; t0w < tiles; t0w += (kThreads / 32 - conv_warps) * kPerWarp) {
-                const int t = min(t0w + lane / kLanes, tiles - 1);       // (the last tile twice rather than none)
-                const int q0 = 4 * (t % qt), j0 = 4 * (t / qt);
-                f32x2 acc[16];
+                for (int g = warp - chain_warps; g * Q < queries; g += kWarps - chain_warps) {
+                    const int q0 = rank + g * Q * ctas;                              // (then every ctas-th)
+                    const int keys = c + min(q0 + (Q - 1) * ctas, b - 1) + 1;        // that the last of them sees
+                    const float* q_row[Q];                                           // (the last query again where there are fewer)
+                    float top[Q], sum[Q];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) acc[e] = 0ull;
-#pragma unroll
-                for (int step = 0; step < 2; ++step) {
-                    const int ch4 = 4 * (gl + kLanes * step);
-                    f32x4 y[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) y[e] = load_pairs(X + (j0 + e) * RS + ch4);      // (rows past S or b: masked below)
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) row_fma<4>(load_pairs(qs + (q0 + a) * RQ + ch4), y, acc + 4 * a);
-                }
-                float v[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) { const float2 f = unpair(acc[e]); v[e] = f.x + f.y; }
-                reduce_lanes<16, kLanes>(v, gl);
-#pragma unroll
-                for (int e = 0; e < kOut; ++e) {
-                    const int idx = gl * kOut + e, q = q0 + (idx >> 2), j = j0 + (idx & 3);
-                    if (q < b && j < S) Ps[j * PS + q] = j <= c + q ? v[e] * sc2 : -INFINITY;
-                }
-            }
-        } else {
-            // ---- 1b. Eq. 6, bias, ReLU: R^T[position][slot]
-            constexpr int kPerWarp = 32 / kLC, kOut = kLC == 16 ? 2 : 1;
-            const int it = (M + 3) / 4, jt = (S + 7) / 8, tiles = it * jt, gl = tid % kLC;
+                    for (int a = 0; a < Q; ++a) { q_row[a] = qs + min(g * Q + a, queries - 1) * RQ; top[a] = -INFINITY; sum[a] = 0.f; }
 #pragma unroll 1
-            for (int t0w = warp * kPerWarp; t0w < tiles; t0w += conv_warps * kPerWarp) {
-                const int t = min(t0w + lane / kLC, tiles - 1);
-                const int i0 = 4 * (t % it), j0 = 8 * (t / it);
-                f32x2 acc[32];
+                    for (int j = lane; j < keys; j += 32) {
+                        const float* x = X + j * RS;
+                        f32x2 acc[Q][2];
 #pragma unroll
-                for (int e = 0; e < 32; ++e) acc[e] = 0ull;
-#pragma unroll 1
-                for (int c4 = gl; c4 < C / 4; c4 += kLC) {
-                    const float* w = Gs + (i0 * k + k - 1) * C + 4 * c4;          // tap t of slot a: w + (a k - t) C
-                    const float* x = X + (j0 - pad) * RS + 4 * c4;
-                    const int slot = k * C;
-                    f32x4 z[8];
+                        for (int a = 0; a < Q; ++a) acc[a][0] = acc[a][1] = 0ull;
+#pragma unroll 4
+                        for (int c4 = 0; c4 < kLD; ++c4) {
+                            const f32x4 y = load_pairs(x + 4 * c4);
 #pragma unroll
-                    for (int e = 0; e < 7; ++e) z[e] = load_pairs(x + e * RS);
-                    x += 7 * RS;
-#pragma unroll 1
-                    for (int tap = 0; tap < k; ++tap, w -= C, x += RS) {
-                        z[7] = load_pairs(x);
+                            for (int a = 0; a < Q; ++a) {
+                                const f32x4 w = load_pairs(q_row[a] + 4 * c4);
+                                fma2(w.lo, y.lo, acc[a][0]);
+                                fma2(w.hi, y.hi, acc[a][1]);
+                            }
+                        }
+                        float s[Q];
 #pragma unroll
-                        for (int a = 0; a < 4; ++a) row_fma<8>(load_pairs(w + a * slot), z, acc + 8 * a);
-#pragma unroll
-                        for (int e = 0; e < 7; ++e) z[e] = z[e + 1];
+                        for (int a = 0; a < Q; ++a) {
+                            const float2 lo = unpair(acc[a][0]), hi = unpair(acc[a][1]);
+                            s[a] = j <= c + q0 + a * ctas ? ((lo.x + lo.y) + (hi.x + hi.y)) * sc2 : -INFINITY;
+                            top[a] = fmaxf(top[a], s[a]);
+                        }
+                        put<Q>(Ps + j * Q, s);
                     }
-                }
-                float v[32];
 #pragma unroll
-                for (int e = 0; e < 32; ++e) { const float2 f = unpair(acc[e]); v[e] = f.x + f.y; }
-                reduce_lanes<32, kLC>(v, gl);
-                const int idx = gl * kOut, i = i0 + (idx >> 3);
-                if (i < M) {
-                    const float bias = P.bias ? P.bias[(P.weights_per_head ? h * M : 0) + i] : 0.f;
+                    for (int a = 0; a < Q; ++a)
 #pragma unroll
-                    for (int e = 0; e < kOut; ++e) {
-                        const int j = j0 + (idx & 7) + e;
-                        if (j < S) Rs[j * MS + i] = i < P.prot ? (j == i ? 1.f : 0.f) : fmaxf(v[e] + bias, 0.f);
+                        for (int of = 16; of; of >>= 1) top[a] = fmaxf(top[a], __shfl_xor_sync(0xffffffffu, top[a], of));
+                    for (int j = lane; j < keys; j += 32) {
+                        float s[Q];
+                        get<Q>(Ps + j * Q, s);
+#pragma unroll
+                        for (int a = 0; a < Q; ++a) sum[a] += s[a] = exp2f(s[a] - top[a]);
+                        put<Q>(Ps + j * Q, s);
                     }
-                }
-            }
-        }
-        __syncthreads();
-        // ---- 2. exponentials of every query's scores: one warp each
-#pragma unroll 1
-        for (int x = warp; x < b; x += kThreads / 32) {
-            float m = -INFINITY;
-            for (int j = lane; j < S; j += 32) m = fmaxf(m, Ps[j * PS + x]);
 #pragma unroll
-            for (int of = 16; of; of >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, of));
-            for (int j = lane; j < S; j += 32) Ps[j * PS + x] = exp2f(Ps[j * PS + x] - m);
-            if (lane == 0) top[x] = m;
-        }
-        __syncthreads();
-        // ---- 3. O = P V / sum P, and the new cache = R [X_K | X_V] / (sum R + eps): kRows rows x four channels per thread
-        {
-            float* next = rows_of(cur ^ 1);
-            auto blend = [&](auto rows_per_thread) {
-                constexpr int kRows = decltype(rows_per_thread)::value;
-                const int o_tiles = (b + kRows - 1) / kRows * kLD, c_tiles = compress ? (M + kRows - 1) / kRows * 2 * kLD : 0;
-#pragma unroll 1
-                for (int t = tid; t < o_tiles + c_tiles; t += kThreads) {
-                    const bool is_o = t < o_tiles;
-                    const int tt = is_o ? t : t - o_tiles;
-                    const int r0 = kRows * (is_o ? tt / kLD : tt / (2 * kLD)), c4 = is_o ? tt % kLD : tt % (2 * kLD), ch4 = is_o ? D + 4 * c4 : 4 * c4;
-                    const int ws = is_o ? PS : MS;
-                    const float* w = (is_o ? Ps : Rs) + r0;
-                    f32x4 acc[kRows];
-                    float sum[kRows];
+                    for (int a = 0; a < Q; ++a)
 #pragma unroll
-                    for (int a = 0; a < kRows; ++a) { acc[a] = f32x4{0ull, 0ull}; sum[a] = 0.f; }
-                    const float* x = X + ch4;
-#pragma unroll 8
-                    for (int j = 0; j < S; ++j, w += ws, x += RS) {
-                        float pr[kRows];
-                        if constexpr (kRows == 4) *reinterpret_cast<float4*>(pr) = load4(w);
-                        else *reinterpret_cast<float2*>(pr) = *reinterpret_cast<const float2*>(w);
+                        for (int of = 16; of; of >>= 1) sum[a] += __shfl_xor_sync(0xffffffffu, sum[a], of);
+                    __syncwarp();
+                    constexpr int kParts = 32 / kLD;                         // lanes that share a channel quad take every other key
+                    const int c4 = lane % kLD, part = lane / kLD;
+                    f32x4 acc[Q];
+#pragma unroll
+                    for (int a = 0; a < Q; ++a) acc[a] = f32x4{0ull, 0ull};
+                    const float *x = X + part * RS + D + 4 * c4, *pr = Ps + part * Q;
+#pragma unroll 4
+                    for (int j = part; j < keys; j += kParts, x += kParts * RS, pr += kParts * Q) {
                         const f32x4 v = load_pairs(x);
+                        float w[Q];
+                        get<Q>(pr, w);
 #pragma unroll
-                        for (int a = 0; a < kRows; ++a) { fma4(pair(pr[a], pr[a]), v, acc[a]); sum[a] += pr[a]; }
+                        for (int a = 0; a < Q; ++a) fma4(pair(w[a], w[a]), v, acc[a]);
                     }
 #pragma unroll
-                    for (int a = 0; a < kRows; ++a) {
-                        const int r = r0 + a;
-                        const float4 v = to_float4(acc[a]);
-                        if (is_o) {
-                            if (r >= b) break;
-                            const float s = 1.f / sum[a];
-                            store4(unit_base_mut<float>(P.o, n, h) + (int64_t)(t0 + r) * P.o.st + 4 * c4, make_float4(v.x * s, v.y * s, v.z * s, v.w * s));
-                            if (P.lse && c4 == 0) P.lse[(int64_t)u * P.L + t0 + r] = (top[r] + log2f(sum[a])) * 0.6931471805599453f;
-                        } else {
-                            if (r >= M) break;
-                            const float s = r < P.prot ? 1.f : 1.f / (sum[a] + P.eps);
-                            store4(next + r * RS + ch4, make_float4(v.x * s, v.y * s, v.z * s, v.w * s));
+                    for (int a = 0; a < Q; ++a) {
+                        float4 v = to_float4(acc[a]);
+                        if (kParts == 2) {
+                            v.x += __shfl_xor_sync(0xffffffffu, v.x, 16); v.y += __shfl_xor_sync(0xffffffffu, v.y, 16);
+                            v.z += __shfl_xor_sync(0xffffffffu, v.z, 16); v.w += __shfl_xor_sync(0xffffffffu, v.w, 16);
+                        }
+                        if (g * Q + a >= queries || part != a % kParts) continue;
+                        const int q = t0 + q0 + a * ctas;
+                        const float s = 1.f / sum[a];
+                        store4(unit_base_mut<float>(P.o, n, h) + (int64_t)q * P.o.st + 4 * c4, make_float4(v.x * s, v.y * s, v.z * s, v.w * s));
+                        if (P.lse && c4 == 0) P.lse[(int64_t)u * P.L + q] = (top[a] + log2f(sum[a])) * 0.6931471805599453f;
+                    }
+                    __syncwarp();
+                }
+            };
+            // as few queries per warp as keep every warp busy once, up to four (a warp's loads of keys and values serve them all)
+            const int warps = kWarps - chain_warps;
+            if (queries <= warps) attend(std::integral_constant<int, 1>{});
+            else if (queries <= 2 * warps) attend(std::integral_constant<int, 2>{});
+            else attend(std::integral_constant<int, 4>{});
+        } else if (compress) {
+            // ---- Eq. 6, bias, ReLU: R^T[position][slot]
+            auto convolve = [&](auto tile_slots, auto tile_positions, auto tile_lanes) {
+                constexpr int TA = decltype(tile_slots)::value, TP = decltype(tile_positions)::value, kL = decltype(tile_lanes)::value;
+                constexpr int kPerWarp = 32 / kL, kAll = TA == 3 ? 4 * TP : TA * TP, kOut = kAll > kL ? kAll / kL : 1;      // (powers of two)
+                const int it = (slots + TA - 1) / TA, jt = (S + TP - 1) / TP, tiles = it * jt, gl = tid % kL;
+                const uint32_t magic = 0xffffffffu / jt + 1;                 // t / jt = the upper half of t magic (jt > 1)
+#pragma unroll 1
+                for (int t0w = warp * kPerWarp; t0w < tiles; t0w += chain_warps * kPerWarp) {
+                    const int t = min(t0w + lane / kL, tiles - 1);           // (the last tile twice rather than none)
+                    const int ti = jt == 1 ? t : __umulhi(t, magic), i0 = TA * ti, j0 = TP * (t - ti * jt);
+                    f32x2 acc[TA * TP];
+#pragma unroll
+                    for (int e = 0; e < TA * TP; ++e) acc[e] = 0ull;
+#pragma unroll 1
+                    for (int c4 = gl; c4 < C / 4; c4 += kL) {
+                        const int slot = k * C;
+                        const float* w = Gs + (i0 * k + k - 1) * C + 4 * c4;          // tap t of slot a: w + (a k - t) C
+                        const float* x = X + (j0 - pad) * RS + 4 * c4;
+                        f32x4 z[TP];                                                  // rows of the window, the first at tap % TP
+#pragma unroll
+                        for (int e = 0; e < TP - 1; ++e) z[e] = load_pairs(x + e * RS);
+                        x += (TP - 1) * RS;
+#pragma unroll 1
+                        for (int tap = 0; tap < k; tap += TP) {
+#pragma unroll
+                            for (int e = 0; e < TP; ++e, w -= C, x += RS) {
+                                if (tap + e >= k) break;
+                                z[(e + TP - 1) % TP] = load_pairs(x);
+#pragma unroll
+                                for (int a = 0; a < TA; ++a) row_fma<TP>(load_pairs(w + a * slot), z, e, acc + TP * a);
+                            }
+                        }
+                    }
+                    float v[kAll];
+#pragma unroll
+                    for (int e = 0; e < kAll; ++e) { const float2 f = unpair(e < TA * TP ? acc[e] : 0ull); v[e] = f.x + f.y; }
+                    reduce_lanes<kAll, kL>(v, gl);
+                    const int idx = gl * kAll / kL, a = i0 + idx / TP, i = i_begin + a;
+                    if (idx < TA * TP && a < slots) {
+                        const float bias = P.bias ? P.bias[(P.weights_per_head ? h * M : 0) + i] : 0.f;
+#pragma unroll
+                        for (int e = 0; e < kOut; ++e) {
+                            const int j = j0 + idx % TP + e;
+                            if (j < S) Rs[j * MS + a] = i < P.prot ? (j == i ? 1.f : 0.f) : fmaxf(v[e] + bias, 0.f);
                         }
                     }
                 }
             };
-            // two rows per thread while that leaves threads over, else four (half the reads per result)
-            if ((b / 2 + (compress ? M : 0)) * kLD <= kThreads) blend(std::integral_constant<int, 2>{});
-            else blend(std::integral_constant<int, 4>{});
+            using Two = std::integral_constant<int, 2>;
+            using Four = std::integral_constant<int, 4>;
+            using Eight = std::integral_constant<int, 8>;
+            using Lanes = std::integral_constant<int, kLC>;
+            using Fewer = std::integral_constant<int, kLC / 2>;
+            if (P.tile == 0) convolve(Four{}, Eight{}, Fewer{});
+            else if (P.tile == 1) convolve(std::integral_constant<int, 3>{}, Eight{}, Fewer{});
+            else if (P.tile == 2) convolve(Two{}, Eight{}, Fewer{});
+            else convolve(Two{}, Four{}, Lanes{});
+            asm volatile("bar.sync 1, %0;" ::"r"(chain_threads) : "memory");
+            // ---- the new rows of this CTA's slots: kRows rows x four channels per group of kParts lanes, which share the positions
+            float* next = rows_of(cur ^ 1) + i_begin * RS;
+            auto blend = [&](auto rows_per_group, auto lanes_per_group) {
+                constexpr int kRows = decltype(rows_per_group)::value, kParts = decltype(lanes_per_group)::value;
+                const int items = (slots + kRows - 1) / kRows * 2 * kLD;
+#pragma unroll 1
+                for (int t0w = 32 * warp; t0w < items * kParts; t0w += chain_threads) {
+                    const int part = lane % kParts, t = min((t0w + lane) / kParts, items - 1);
+                    const int r0 = kRows * (t / (2 * kLD)), ch4 = 4 * (t % (2 * kLD));
+                    f32x4 acc[kRows];
+                    float sum[kRows];
+#pragma unroll
+                    for (int a = 0; a < kRows; ++a) { acc[a] = f32x4{0ull, 0ull}; sum[a] = 0.f; }
+                    const float *w = Rs + part * MS + r0, *x = X + part * RS + ch4;
+#pragma unroll 4
+                    for (int j = part; j < S; j += kParts, w += kParts * MS, x += kParts * RS) {
+                        float r[kRows];
+                        get<kRows>(w, r);
+                        const f32x4 v = load_pairs(x);
+#pragma unroll
+                        for (int a = 0; a < kRows; ++a) { fma4(pair(r[a], r[a]), v, acc[a]); sum[a] += r[a]; }
+                    }
+                    float v[4 * kRows];
+#pragma unroll
+                    for (int a = 0; a < kRows; ++a) {
+                        const float4 f = to_float4(acc[a]);
+                        v[4 * a] = f.x; v[4 * a + 1] = f.y; v[4 * a + 2] = f.z; v[4 * a + 3] = f.w;
+#pragma unroll
+                        for (int m = kParts / 2; m; m >>= 1) sum[a] += __shfl_xor_sync(0xffffffffu, sum[a], m);
+                    }
+                    reduce_lanes<4 * kRows, kParts>(v, part);
+                    constexpr int kOut = 4 * kRows / kParts, kVec = kOut < 4 ? kOut : 4;      // results of a lane, of one store
+                    const int first = part * kOut;
+#pragma unroll
+                    for (int e = 0; e < kOut; e += kVec) {
+                        const int a = (first + e) / 4, r = r0 + a;
+                        float own = sum[0];                        // (no indexing by a variable)
+#pragma unroll
+                        for (int y = 1; y < kRows; ++y) own = a == y ? sum[y] : own;
+                        if (r >= slots) break;
+                        const float s = i_begin + r < P.prot ? 1.f : 1.f / (own + P.eps);
+#pragma unroll
+                        for (int y = 0; y < kVec; ++y) v[e + y] *= s;
+                        float* dst = next + r * RS + ch4 + (first + e) % 4;
+                        if (ctas > 1) store_everywhere<kVec>(dst, v + e, rank, ctas);
+                        else {
+#pragma unroll
+                            for (int y = 0; y < kVec; ++y) dst[y] = v[e + y];
+                        }
+                    }
+                }
+            };
+            // four rows per group where there are as many, and as many lanes per group as there are threads for
+            auto lanes = [&](auto rows_per_group) {
+                const int items = (slots + decltype(rows_per_group)::value - 1) / decltype(rows_per_group)::value * 2 * kLD;
+                if (8 * items <= chain_threads) blend(rows_per_group, Eight{});
+                else if (4 * items <= chain_threads) blend(rows_per_group, Four{});
+                else if (2 * items <= chain_threads) blend(rows_per_group, Two{});
+                else blend(rows_per_group, std::integral_constant<int, 1>{});
+            };
+            if (slots > 2) lanes(Four{});
+            else lanes(Two{});
         }
         if (compress) {
             cur ^= 1;
@@ -307,10 +424,11 @@ __global__ void __launch_bounds__(kThreads, 1) small_loop_kernel(const __grid_co
         } else {
             c = S;                                          // fill: the chunk's rows are where they belong
         }
+        cp_async_wait<0>();
+        everybody();
     }
-    __syncthreads();
     const float* cache = rows_of(cur);
-    for (int x = tid; x < c * 2 * kLD; x += kThreads) {
+    for (int x = rank * kThreads + tid; x < c * 2 * kLD; x += ctas * kThreads) {
         const int r = x / (2 * kLD), q4 = x % (2 * kLD);
         const View& v = q4 < kLD ? P.k_cache : P.v_cache;
         store4(unit_base_mut<float>(v, n, h) + (int64_t)r * v.st + 4 * (q4 % kLD), load4(cache + r * RS + 4 * q4));
@@ -319,27 +437,55 @@ __global__ void __launch_bounds__(kThreads, 1) small_loop_kernel(const __grid_co
 
 template <int D, int kLC>
 int launch_loop(const LoopParams& P, int units, size_t smem, cudaStream_t st) {
-    static bool done[64] = {};
-    if (!smem_limit(small_loop_kernel<D, kLC>, kMaxSmem, done)) return -1;
-    return launch_after(small_loop_kernel<D, kLC>, dim3(units), dim3(kThreads), smem, st, P) ? 1 : -1;
+    static ClusterKernel state;
+    return launch_clusters(state, small_loop_kernel<D, kLC>, kMaxSmem, P.ctas, units, kThreads, smem, st, P) ? 1 : -1;
+}
+
+ClusterKernel loop_state;      // of the kernel that is asked how many clusters fit (all forms need an SM per CTA)
+
+struct LoopPlan {
+    int ctas, chain_warps, tile;     // (ctas 0: not this way)
+};
+
+// The plan, and the rule: fp32, [cache; chunk] in one SM's shared memory, and a chunk estimated faster than as launches over the whole
+// chip. Both estimates (us per chunk) are fitted to 44 shapes on a B200, every cluster size each, half of them within 10 % of the one
+// for clusters; the launches are slowest where a tile's channels and taps are many. Measured, launches / this, us per call: 256 tokens of
+// one unit, M = B = 16, d = 64, k = 5 263 / 41; of 148 units 383 / 69; 777 tokens of 8 units, M = 48, B = 100 180 / 72; 85 tokens of one unit,
+// M = B = 16, d = 128, k = 25 248 / 31; 349 tokens of 16 units, M = B = 64, k = 25 513 / 170. In no shape that fits were the launches faster.
+LoopPlan loop_plan(const lococo_handle* h, int L, int B) {
+    const lococo_config& c = h->cfg;
+    LoopPlan best{0, 0, 0};
+    if (c.dtype != LOCOCO_F32) return best;
+    B = std::min(B, L);
+    const double S = (double)c.M + B, keys = c.M + 0.5 * B, d2 = 2.0 * c.head_dim, taps = (double)c.c_in * c.k;
+    if (2.0 * S * d2 * 4 > kMaxSmem) return best;
+    double least = 11.0 + 0.012 * taps + h->units * (c.M * S * (taps + d2) + B * keys * d2) / (kSMs * 150000.0);
+    for (int ctas = 1; ctas <= std::min(kMaxCluster, c.M); ctas = ctas < 8 ? 2 * ctas : ctas + 1) {
+        const int slots = (c.M + ctas - 1) / ctas, queries = (B + ctas - 1) / ctas, clusters = resident_clusters(loop_state, small_loop_kernel<64, 16>, kMaxSmem, ctas, kThreads);
+        const double conv = slots * S * taps, blends = slots * S * d2, attention = queries * keys * d2;
+        LoopPlan p{ctas, std::min(12, std::max(4, 2 * (int)(0.5 * kWarps * (conv + blends) / (conv + blends + 1.3 * attention) + 0.5))), 3};
+        const LoopLayout lay = loop_layout(c.head_dim, c.M, B, c.k, c.c_in, ctas, kWarps - p.chain_warps);
+        if (clusters == 0 || (double)slots * taps * 4 > kMaxSmem || (size_t)lay.total * 4 > kMaxSmem) continue;
+        const double t = (h->units + clusters - 1) / clusters * (2.4 + 0.025 * ctas + conv / 109e3 + blends / 240e3 + attention / 91e3);
+        if (t >= least) continue;
+        least = t;
+        // Tiles of 2 x 4 while that is one round of the chain's lanes; else 8 positions wide, of as many slots as waste least
+        const int lanes = c.head_dim == 64 && c.c_in == 64 ? 16 : 32, threads = 32 * p.chain_warps;
+        if ((slots + 1) / 2 * (((int)S + 3) / 4) * lanes > threads) {
+            double cost = 1e30;
+            for (int a = 4; a >= 2; --a) {
+                const double rounds = ((slots + a - 1) / a * (((int)S + 7) / 8) * (lanes / 2) + threads - 1) / threads;
+                if (rounds * (a + 0.7) < cost) { cost = rounds * (a + 0.7); p.tile = 4 - a; }
+            }
+        }
+        best = p;
+    }
+    return best;
 }
 
 }  // namespace
 
-// The rule: fp32, everything in one SM's shared memory, and one block per unit is estimated faster than three launches per
-// chunk over the whole chip. A block does about 45 FMAs per cycle, a third of an SM's rate (M = B = 16, d = 64, k = 5: 4.65 us per
-// chunk by the rule, 4.7 measured); the launches cost about 13 us per chunk besides 55 FMAs per cycle and SM.
-bool simt_loop_preferred(const lococo_handle* h, int L, int B) {
-    const lococo_config& c = h->cfg;
-    if (c.dtype != LOCOCO_F32) return false;
-    const LoopLayout lay = loop_layout(c.head_dim, c.M, std::min(B, L), c.k, c.c_in);
-    const double floats = (double)((c.M + 3) / 4 * 4) * c.k * c.c_in + 4.0 * ((double)c.M + std::min(B, L) + c.k) * c.head_dim;
-    if (floats * 4 > kMaxSmem || lay.total < 0 || (size_t)lay.total * 4 > kMaxSmem) return false;
-    const double S = c.M + std::min(B, L), b = std::min(B, L);
-    const double fma = (double)c.M * S * c.c_in * c.k + 2.0 * c.M * S * c.head_dim + 2.0 * b * (c.M + b) * c.head_dim;
-    const double one = 1.2 + (h->units + kSMs - 1) / kSMs * fma / 45.0 / 1900.0, many = 13.0 + h->units * fma / (kSMs * 55.0) / 1900.0;
-    return one < many;
-}
+bool simt_loop_preferred(const lococo_handle* h, int L, int B) { return loop_plan(h, L, B).ctas > 0; }
 
 int simt_loop(lococo_handle* h, View q, View k, View v, int L, int B, View o, View kc, View vc, int c0, char* saved, size_t snap_step,
               size_t snap_all, cudaStream_t st) {
@@ -352,25 +498,15 @@ int simt_loop(lococo_handle* h, View q, View k, View v, int L, int B, View o, Vi
     P.bias = h->has_bias ? reinterpret_cast<const float*>(h->ws + h->off_bias) : nullptr;
     P.eps = c.norm_eps;
     P.scale = h->scale;
-    {
-        // warps for the convolution: where the slower of the two kinds of tiles is done first (a tile's time is about its
-        // loads: k + 7 rows and 4 k weights of a 4 x 8 tile, 8 rows of a 4 x 4 score tile, 10 for the sums and the store)
-        const int S = P.M + P.B, conv_lanes = std::min(P.c_in / 4, 32), warps = kThreads / 32;
-        const int conv = ((P.M + 3) / 4 * ((S + 7) / 8) * conv_lanes + 31) / 32, conv_cost = (5 * P.k_taps + 7) * std::max(1, P.c_in / 128) + 20;
-        const int score = ((P.B + 3) / 4 * ((S + 3) / 4) * (P.d / 8) + 31) / 32, score_cost = 16 + 10;
-        int best = 1 << 30;
-        for (int w = 1; w < warps; ++w) {
-            const int t = std::max((conv + w - 1) / w * conv_cost, (score + warps - w - 1) / (warps - w) * score_cost);
-            if (t < best) { best = t; P.conv_warps = w; }
-        }
-    }
+    const LoopPlan plan = loop_plan(h, L, B);
+    P.ctas = plan.ctas; P.chain_warps = plan.chain_warps; P.tile = plan.tile;
     if (saved) {
         P.snap_k = reinterpret_cast<float*>(saved);
         P.snap_v = reinterpret_cast<float*>(saved + snap_all);
         P.snap_step = (int64_t)(snap_step / sizeof(float));
         P.lse = reinterpret_cast<float*>(saved + 2 * snap_all);
     }
-    const size_t smem = (size_t)loop_layout(P.d, P.M, P.B, P.k_taps, P.c_in).total * 4;
+    const size_t smem = (size_t)loop_layout(P.d, P.M, P.B, P.k_taps, P.c_in, P.ctas, kWarps - P.chain_warps).total * 4;
     prof_begin(&h->prof, PROF_SEQUENCE, st);
     const int r = P.d == 128 ? launch_loop<128, 32>(P, h->units, smem, st)
                 : P.c_in == 64 ? launch_loop<64, 16>(P, h->units, smem, st) : launch_loop<64, 32>(P, h->units, smem, st);

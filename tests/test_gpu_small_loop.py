@@ -66,3 +66,45 @@ def test_the_loop_is_timed_on_request():
     ms, launches = ctx.profile_read(3)
     ctx.profile(False)
     assert launches == 1 and 0 < ms < 100
+
+
+@pytest.mark.parametrize("batch,heads,d,M,B,L,k,c_mult,prot", [
+    (1, 1, 64, 17, 33, 150, 7, 1, 0),         # the widest clusters: CTAs of one and of two slots, of two and of three queries
+    (1, 1, 64, 3, 40, 130, 9, 2, 1),          # fewer slots than CTAs would fit
+    (3, 4, 64, 30, 21, 104, 5, 1, 5),         # CTAs with and without protected slots
+    (2, 20, 128, 13, 9, 48, 3, 1, 0),         # clusters of a few CTAs; fill steps first
+    (5, 30, 64, 18, 26, 120, 5, 1, 0),        # a CTA per unit
+    (1, 2, 64, 65, 30, 190, 11, 1, 0),        # tiles of 8 positions; fill steps whose chunks several CTAs read
+])
+def test_small_loop_clusters(batch, heads, d, M, B, L, k, c_mult, prot):
+    # Snapshots on (the gradients' inputs), so that what every CTA holds of the cache is seen after every chunk.
+    from oracle import lococo_oracle as orc
+    from paper_2406_05317_b200 import api
+    w = wl.Workload("small_loop_clusters", 63, batch=batch, heads=heads, d=d, M=M, B=B, k=k, L=L, dtype="f32", weights_per_head=True,
+                    qkv_scale=1.0, g_std=0.05, c_in_mult=c_mult)
+    ctx = api.Lococo(batch, heads, d, M, k, B, dtype=torch.float32, c_in=w.c_in, weights_per_head=True)
+    G, bias = wl.make_weights(w, with_bias=True)
+    ctx.set_weights(to_device(G, "f32"), to_device(bias, "f32"))
+    ctx.set_protected_slots(prot)
+    Q, K, V = wl.make_qkv(w)
+    dQ, dK, dV = (to_device(x, "f32") for x in (Q, K, V))
+    O, Kc, Vc = torch.empty_like(dQ), torch.zeros(batch, heads, M, d, device="cuda"), torch.zeros(batch, heads, M, d, device="cuda")
+    saved = torch.zeros(ctx.saved_bytes(L, B), dtype=torch.uint8, device="cuda")
+    launches = ctx.launch_count()
+    c = ctx.process_sequence(dQ, dK, dV, B, O, Kc, Vc, 0, saved)
+    assert ctx.launch_count() - launches == 1
+    torch.cuda.synchronize()
+    chunks, step = -(-L // B), batch * heads * M * d
+    size = (chunks * step * 4 + 255) // 256 * 256
+    snaps = [saved[i * size:].view(torch.float32)[:chunks * step].view(chunks, batch, heads, M, d).cpu().numpy() for i in range(2)]
+    for u in (0, batch * heads // 2, batch * heads - 1):
+        n, h = divmod(u, heads)
+        Or, Kr, Vr, cr, _, sK, sV, sc = orc.process_sequence(Q[n, h], K[n, h], V[n, h], G[h], B, bias=bias[h], protected=prot, want_snapshots=True)
+        assert c == cr
+        assert_close(to_host(O)[n, h], Or, "f32", "O")
+        assert_close(to_host(Kc)[n, h], Kr, "f32", "K cache")
+        assert_close(to_host(Vc)[n, h], Vr, "f32", "V cache")
+        for i in range(chunks):
+            for got, want in zip(snaps, (sK, sV)):
+                if sc[i]:
+                    assert_close(got[i, n, h, :sc[i]], want[i, :sc[i]], "f32", f"cache before chunk {i}")
