@@ -89,3 +89,12 @@ def test_no_second_round_of_clusters():
         return best
 
     assert max(step_us(34), step_us(37)) < 1.4 * step_us(32)
+
+
+@pytest.mark.parametrize("batch,heads,k,per_head,prot", [
+    (1, 149, 1, False, 0),     # the fewest units that share SMs; one tap: fewer weight pieces than ring stages
+    (3, 99, 27, True, 3),      # one unit more than run at the same time; the most taps
+    (7, 43, 5, False, 128),    # 301 units; every slot kept
+])
+def test_two_ctas_per_sm(batch, heads, k, per_head, prot):
+    test_generation_kernel(batch, heads, k, per_head, prot)
