@@ -107,7 +107,8 @@ View bdev(const lococo_tensor& t, int64_t tokens, size_t elt) {
 }
 
 struct Scratch {
-    size_t gK, gV, parts, dA, delta, tensor, total;
+    size_t gK, gV, parts, dA, delta, tensor, group, total;
+    int group_chunks;          // chunks that one go of the CUDA cores can take (0: a step at a time)
 };
 
 Scratch scratch_layout(const lococo_handle* h, int L, int B) {
@@ -124,6 +125,11 @@ Scratch scratch_layout(const lococo_handle* h, int L, int B) {
     } else {
         s.parts = take(simt_backward_parts_floats(h->units, c.M, B, c.head_dim) * sizeof(float));
         s.dA = take(units * c.M * ((Smax + 3) / 4 * 4) * sizeof(float));
+        // (in the place of what single steps need: a call takes the one way or the other)
+        size_t floats = 0;
+        s.group = s.parts;
+        s.group_chunks = simt_group_chunks(h, L, B, &floats);
+        off = std::max(off, s.group + align256(floats * sizeof(float)));
     }
     s.total = off;
     return s;
@@ -173,19 +179,52 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
     const char* sv = static_cast<const char*>(saved);
     const float* lse_all = reinterpret_cast<const float*>(sv + 2 * snap_all);
 
+    float* delta = reinterpret_cast<float*>(sc + sl.delta);
+
+    // the CUDA cores take several chunks at a time where those of one would not fill the chip
+    BwdGroup G{};
+    if (sl.group_chunks) {
+        const lococo_tensor snap{const_cast<char*>(sv), (int64_t)cfg.heads * cfg.M * cfg.head_dim, (int64_t)cfg.M * cfg.head_dim, (int64_t)cfg.head_dim};
+        lococo_tensor snapV = snap;
+        snapV.ptr = const_cast<char*>(sv) + snap_all;
+        BwdStep& p = G.first;
+        p.xk = CatView{bdev(snap, 0, e), bdev(K, 0, e), 0, 0};
+        p.xv = CatView{bdev(snapV, 0, e), bdev(V, 0, e), 0, 0};
+        p.q = bdev(Q, 0, e); p.o = bdev(O, 0, e); p.d_o = bdev(dO, 0, e);
+        p.dq = bdev(dQ, 0, e); p.dk = bdev(dK, 0, e); p.dv = bdev(dV, 0, e);
+        p.heads = cfg.heads; p.units = h->units; p.d = cfg.head_dim; p.M = cfg.M; p.k = cfg.k; p.c_in = cfg.c_in;
+        p.weights_per_head = cfg.weights_per_head;
+        p.g_reverse = h->ws + h->off_greverse;
+        p.scale = h->scale;
+        p.lse = lse_all; p.lse_stride = L;
+        p.delta = delta; p.delta_stride = L;
+        p.dG = dG; p.dbias = dbias;
+        G.L = L; G.B = std::min(B, L); G.c0 = cache_len_in;
+        G.snap_step = (int64_t)(snap_step / e);
+        G.S = cfg.M + G.B; G.Sr = (G.S + 3) / 4 * 4;
+        p.Sr = G.Sr;
+        G.g_packed = h->ws + h->off_gpack;
+        G.bias = h->has_bias ? reinterpret_cast<const float*>(h->ws + h->off_bias) : nullptr;
+        G.eps = cfg.norm_eps; G.prot = h->prot;
+        G.gk_final = bdev(dKc_final, 0, e); G.gv_final = bdev(dVc_final, 0, e);
+        G.gK = gK; G.gV = gV;
+    }
+    const bool grouped = sl.group_chunks && simt_group_supported(G);
     char* tb = tensor_backward_supported(h) ? sc + sl.tensor : nullptr;
     if (tb) {
         const int r = tensor_backward_prepare(h, B, tb, st);
         if (r < 0) return LOCOCO_ERR_CUDA;
         h->launches += r;
     }
-    int launched_n = cfg.dtype == LOCOCO_F32
+    int launched_n = 0;
+    if (!grouped) {      // (a group's chain reads the caller's tensors)
+        launched_n = cfg.dtype == LOCOCO_F32
                          ? init_g<float>(bdev(dKc_final, 0, e), bdev(dVc_final, 0, e), gK, gV, cfg.heads, h->units, cfg.M, cfg.head_dim, st)
                          : init_g<__nv_bfloat16>(bdev(dKc_final, 0, e), bdev(dVc_final, 0, e), gK, gV, cfg.heads, h->units, cfg.M,
                                                  cfg.head_dim, st);
-    if (launched_n < 0) return LOCOCO_ERR_CUDA;
-    h->launches += launched_n;
-    float* delta = reinterpret_cast<float*>(sc + sl.delta);
+        if (launched_n < 0) return LOCOCO_ERR_CUDA;
+        h->launches += launched_n;
+    }
     launched_n = cfg.dtype == LOCOCO_F32 ? deltas<float>(bdev(O, 0, e), bdev(dO, 0, e), delta, cfg.heads, h->units, L, cfg.head_dim, st)
                                          : deltas<__nv_bfloat16>(bdev(O, 0, e), bdev(dO, 0, e), delta, cfg.heads, h->units, L, cfg.head_dim, st);
     if (launched_n < 0) return LOCOCO_ERR_CUDA;
@@ -199,7 +238,15 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
         c_before[n] = c;
         c = c + b <= cfg.M ? c + b : cfg.M;
     }
-    for (int n = n_chunks - 1; n >= 0; --n) {
+    for (int n = n_chunks; grouped && n > 0; n -= G.count) {
+        G.count = std::min(n, sl.group_chunks);
+        G.n0 = n - G.count;
+        simt_group_layout(G, reinterpret_cast<float*>(sc + sl.group));
+        const int r = simt_backward_group(G, st);
+        if (r < 0) return LOCOCO_ERR_CUDA;
+        h->launches += r;
+    }
+    for (int n = grouped ? -1 : n_chunks - 1; n >= 0; --n) {
         const int t0 = n * B, b = std::min(B, L - t0), c = c_before[n];
         lococo_tensor snapK{const_cast<char*>(sv) + (size_t)n * snap_step, (int64_t)cfg.heads * cfg.M * cfg.head_dim,
                             (int64_t)cfg.M * cfg.head_dim, (int64_t)cfg.head_dim};
@@ -221,7 +268,7 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
         p.dA = reinterpret_cast<float*>(sc + sl.dA);
         p.Sr = (p.S + 3) / 4 * 4;
         p.delta = delta + t0; p.delta_stride = L;
-        p.gK = gK; p.gV = gV;
+        p.gK = gK; p.gV = gV; p.g_st = cfg.head_dim;
         p.dG = dG; p.dbias = dbias;
         CompressParams f{};
         f.xk = p.xk; f.xv = p.xv;

@@ -38,6 +38,9 @@ __device__ __forceinline__ void axpy4(float s, const float4& x, float4& y) {
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16u : 0u) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 4u : 0u) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -174,6 +177,28 @@ __device__ __forceinline__ float4 to_float4(const f32x4& v) {
     return make_float4(a.x, a.y, b.x, b.y);
 }
 
+// Sums of v[0..N-1] over the L lanes of a group (powers of two); lane l of the group is left with max(1, N / L) results in
+// v[0..], from index l * N / L on (L > N: every L / N lanes hold the same one).
+template <int N, int L>
+__device__ __forceinline__ void reduce_lanes(float (&v)[N], int lane) {
+    int n = N;
+#pragma unroll
+    for (int m = L / 2; m > 0; m >>= 1) {
+        if (n == 1) {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
+            continue;
+        }
+        n >>= 1;
+        const bool up = lane & m;
+#pragma unroll
+        for (int e = 0; e < N / 2; ++e) {
+            if (e >= n) break;
+            const float send = up ? v[e] : v[e + n], keep = up ? v[e + n] : v[e];
+            v[e] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+    }
+}
+
 // Barrier of a group of 128 threads of a block (group g of a block of several, or the whole block: g = 0).
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g) : "memory"); }
 
@@ -187,6 +212,12 @@ struct ConvAcc {
             for (int y = 0; y < 4; ++y) v[x][y] = 0ull;
     }
     __device__ __forceinline__ float get(int x, int y) const { const float2 f = unpair(v[x >> 1][y]); return (x & 1) ? f.y : f.x; }
+    __device__ __forceinline__ void add(const ConvAcc& o) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) { const float2 a = unpair(v[x][y]), b = unpair(o.v[x][y]); v[x][y] = pair(a.x + b.x, a.y + b.y); }
+    }
 };
 
 // A 1-D convolution of many channels in fp32, one tile of OT outputs x PT positions per group of 128 threads (`tid` within the
@@ -207,9 +238,10 @@ struct WindowConv {
     // thread's outputs: two groups of four consecutive ones, half a tile apart
     __device__ static __forceinline__ int out_index(int ti, int x) { return x < 4 ? 4 * ti + x : OT / 2 + 4 * ti + x - 4; }
 
-    template <typename Input>
+    // kSums: `total` takes sums of sixteen channels at a time (a long contraction's rounding errors grow with the longest chain of additions).
+    template <bool kSums = false, typename Input>
     __device__ static __forceinline__ void run(const T* w, int n_in, int n_out, int k, int o0, int x0, int c_begin, int c_end, const Input& in,
-                                               float* smem, ConvAcc& acc, int tid, int bar) {
+                                               float* smem, ConvAcc& acc, int tid, int bar, ConvAcc* total = nullptr) {
         const int ti = tid % TI, tj = tid / TI;
         const int rows = PT + k - 1, ZW = PT + (k + 2) / 4 * 4 + 4;
         float* Ws = smem;                       // [2][8][8][OT]
@@ -308,6 +340,10 @@ struct WindowConv {
                         taps(z, wp + (c * 8 + t4) * OT, nt - t4);
                     }
                 }
+            }
+            if (kSums && piece == tap_pieces - 1 && (((chunk - c_begin) & 1) || step + 1 == steps)) {
+                total->add(acc);
+                acc.clear();
             }
             if (fetch) put_inputs(chunk + 1);   // (the buffer this chunk's predecessor used: its readers passed the barrier above)
         }

@@ -24,12 +24,14 @@ using namespace simt;
 //   s = F1 S1^T, dp = F2 S2^T     (F1, S1: keys and queries; F2, S2: values and output gradients)
 //   p = exp(scale s - lse), ds = scale p (dp - delta)     under the causal mask
 //   dF1 += ds S1,  dF2 += p S2 (keys' side only)
-// A thread computes 4 x 2 scores and 4 rows x D/16 channels of each gradient.
+// A thread computes 4 x 2 scores and 4 rows x D/16 channels of each gradient. The next tile is on its way while one is computed
+// (fp32: asynchronous copies into the other of two stages).
 template <int D>
 struct GradSmem {
     static constexpr int kRow = D + 4;
     static constexpr int kTile = 32 * kRow;
-    static constexpr int kGroup = 2 * kTile + 2 * 32 * 36 + 2 * 32;
+    static constexpr int kStage = 2 * kTile + 2 * 32;                 // streamed rows, and lse and delta of queries
+    static constexpr int kGroup = 2 * kStage + 2 * 32 * 36;           // two stages
     static constexpr int kFloats = 2 * kTile + 2 * kGroup;
 };
 
@@ -37,9 +39,8 @@ template <typename T, int D, bool kKeys>
 __device__ __forceinline__ void attention_grad(const BwdStep& p, float* dx_attn, float* smem, int tile, int u) {
     constexpr int RS = GradSmem<D>::kRow, NC = D / 64;
     const int group = threadIdx.x >> 7;
-    float *F1 = smem, *F2 = F1 + GradSmem<D>::kTile, *S1 = F2 + GradSmem<D>::kTile + group * GradSmem<D>::kGroup, *S2 = S1 + GradSmem<D>::kTile;
-    float *Ds = S2 + GradSmem<D>::kTile, *Ps = Ds + 32 * 36;        // [32 fixed rows][32 streamed rows], row stride 36
-    float *lse_s = Ps + 32 * 36, *delta_s = lse_s + 32;             // of the 32 queries at hand
+    float *F1 = smem, *F2 = F1 + GradSmem<D>::kTile, *stages = F2 + GradSmem<D>::kTile + group * GradSmem<D>::kGroup;
+    float *Ds = stages + 2 * GradSmem<D>::kStage, *Ps = Ds + 32 * 36;        // [32 fixed rows][32 streamed rows], row stride 36
     const int n = u / p.heads, h = u % p.heads;
     const int tid = threadIdx.x & 127, ts = tid & 15, tf = tid >> 4;
     const int f0 = tile * 32;
@@ -48,25 +49,28 @@ __device__ __forceinline__ void attention_grad(const BwdStep& p, float* dx_attn,
     auto stage = [&](bool keys, int r0, float* a, float* b, int first, int threads) {
         for (int e = first; e < 32 * (D / 4); e += threads) {
             const int r = e / (D / 4), q4 = e % (D / 4), row = r0 + r;
-            float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
-            if (row < (keys ? p.S : p.b)) {
-                va = load4((keys ? cat_row<T>(p.xk, n, h, row) : unit_base<T>(p.q, n, h) + (int64_t)row * p.q.st) + 4 * q4);
-                vb = load4((keys ? cat_row<T>(p.xv, n, h, row) : unit_base<T>(p.d_o, n, h) + (int64_t)row * p.d_o.st) + 4 * q4);
+            const bool live = row < (keys ? p.S : p.b);
+            const T* va = live ? (keys ? cat_row<T>(p.xk, n, h, row) : unit_base<T>(p.q, n, h) + (int64_t)row * p.q.st) + 4 * q4 : unit_base<T>(p.q, n, h);
+            const T* vb = live ? (keys ? cat_row<T>(p.xv, n, h, row) : unit_base<T>(p.d_o, n, h) + (int64_t)row * p.d_o.st) + 4 * q4 : unit_base<T>(p.q, n, h);
+            if constexpr (sizeof(T) == 4) {
+                cp_async16(a + r * RS + 4 * q4, va, live);
+                cp_async16(b + r * RS + 4 * q4, vb, live);
+            } else {
+                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+                *reinterpret_cast<float4*>(a + r * RS + 4 * q4) = live ? load4(va) : zero;
+                *reinterpret_cast<float4*>(b + r * RS + 4 * q4) = live ? load4(vb) : zero;
             }
-            *reinterpret_cast<float4*>(a + r * RS + 4 * q4) = va;
-            *reinterpret_cast<float4*>(b + r * RS + 4 * q4) = vb;
         }
     };
-    auto stage_vectors = [&](int r0) {
-        if (tid < 32) {
-            const int r = r0 + tid;
-            lse_s[tid] = r < p.b ? p.lse[(int64_t)u * p.lse_stride + r] * 1.4426950408889634f : 0.f;
-            delta_s[tid] = r < p.b ? p.delta[(int64_t)u * p.delta_stride + r] : 0.f;
+    auto stage_vectors = [&](int r0, float* to) {      // lse, delta
+        if (tid < 64) {
+            const int r = r0 + (tid & 31);
+            const float* src = tid < 32 ? p.lse + (int64_t)u * p.lse_stride : p.delta + (int64_t)u * p.delta_stride;
+            cp_async4(to + tid, r < p.b ? src + r : src, r < p.b);
         }
     };
     stage(kKeys, f0, F1, F2, threadIdx.x, 256);
-    if (!kKeys) stage_vectors(f0);
-    __syncthreads();
+    if (!kKeys) stage_vectors(f0, stages + 2 * GradSmem<D>::kTile);
     f32x4 g1[4][NC], g2[4][NC];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -75,12 +79,29 @@ __device__ __forceinline__ void attention_grad(const BwdStep& p, float* dx_attn,
     // streamed rows that meet the fixed ones: queries from the first that sees key f0, keys up to the last query's limit
     const int s_begin = kKeys ? max(0, f0 - p.c) / 32 * 32 : 0;
     const int s_end = kKeys ? p.b : p.c + min(f0 + 31, p.b - 1) + 1;
+    auto stream = [&](int s0, int which) {
+        float* to = stages + which * GradSmem<D>::kStage;
+        stage(!kKeys, s0, to, to + GradSmem<D>::kTile, tid, 128);
+        if (kKeys) stage_vectors(s0, to + 2 * GradSmem<D>::kTile);
+    };
+    const int s_first = s_begin + 32 * group;
+    if (s_first < s_end) stream(s_first, 0);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    int at = 0;
 #pragma unroll 1
-    for (int s0 = s_begin + 32 * group; s0 < s_end; s0 += 64) {
-        group_sync(1 + group);
-        stage(!kKeys, s0, S1, S2, tid, 128);
-        if (kKeys) stage_vectors(s0);
-        group_sync(1 + group);
+    for (int s0 = s_first; s0 < s_end; s0 += 64, at ^= 1) {
+        if (s0 > s_first) {
+            cp_async_wait<0>();
+            group_sync(1 + group);                                  // this tile is there, and nobody reads the other stage any more
+        }
+        if (s0 + 64 < s_end) {
+            stream(s0 + 64, at ^ 1);
+            cp_async_commit();
+        }
+        const float *S1 = stages + at * GradSmem<D>::kStage, *S2 = S1 + GradSmem<D>::kTile;
+        const float *lse_s = (kKeys ? S1 : stages) + 2 * GradSmem<D>::kTile, *delta_s = lse_s + 32;      // of the 32 queries at hand
         f32x2 s2[4][2], dp2[4][2];                                  // sums over the even and over the odd channels
 #pragma unroll
         for (int a = 0; a < 4; ++a) s2[a][0] = s2[a][1] = dp2[a][0] = dp2[a][1] = 0ull;
@@ -115,7 +136,7 @@ __device__ __forceinline__ void attention_grad(const BwdStep& p, float* dx_attn,
             for (int b = 0; b < 2; ++b) {
                 const int fr = 4 * tf + a, sr = ts + 16 * b;
                 const int key = kKeys ? f0 + fr : s0 + sr, query = kKeys ? s0 + sr : f0 + fr, q = kKeys ? sr : fr;
-                const float pr = (key < p.S && query < p.b && key <= p.c + query) ? exp2f(fmaf(s[a][b], sc2, -lse_s[q])) : 0.f;
+                const float pr = (key < p.S && query < p.b && key <= p.c + query) ? exp2f(fmaf(s[a][b], sc2, -1.4426950408889634f * lse_s[q])) : 0.f;
                 Ds[fr * 36 + sr] = pr * (dp[a][b] - delta_s[q]) * p.scale;
                 if (kKeys) Ps[fr * 36 + sr] = pr;
             }
@@ -147,7 +168,7 @@ __device__ __forceinline__ void attention_grad(const BwdStep& p, float* dx_attn,
     }
     // the second group's sums through its own buffers
     group_sync(1 + group);
-    float *G1 = F2 + GradSmem<D>::kTile + GradSmem<D>::kGroup, *G2 = G1 + GradSmem<D>::kTile;
+    float *G1 = F2 + GradSmem<D>::kTile + GradSmem<D>::kGroup, *G2 = G1 + GradSmem<D>::kTile;      // (its stages)
     if (group == 1) {
 #pragma unroll
         for (int a = 0; a < 4; ++a)
@@ -184,9 +205,10 @@ __device__ __forceinline__ void attention_grad(const BwdStep& p, float* dx_attn,
 // ------------------------------------------------------------------ dw
 // dw[u][i][j] = <gK[u][i], XK[j]> + <gV[u][i], XV[j]>: 64 slots x 64 positions per group of 128 threads (8 x 4 each), sixteen
 // channels per stage, both operands transposed on their way into shared memory.
+// `out(u, i, j, v)` takes v = dw[u][i][j .. j + 3].
 constexpr int kDwFloats = 2 * 16 * 68;
-template <typename T>
-__device__ __forceinline__ void dw_body(const BwdStep& p, float* smem, int block, int tid, int group) {
+template <typename T, typename Out>
+__device__ __forceinline__ void dw_body(const BwdStep& p, float* smem, int block, int tid, int group, const Out& out) {
     float (*As)[68] = reinterpret_cast<float (*)[68]>(smem), (*Xs)[68] = As + 16;
     const int pos_tiles = (p.S + 63) / 64, slot_tiles = (p.M + 63) / 64;
     const int j0 = block % pos_tiles * 64; block /= pos_tiles;
@@ -204,7 +226,7 @@ __device__ __forceinline__ void dw_body(const BwdStep& p, float* smem, int block
         const int c0 = (is_v ? ch0 - p.d : ch0) + 8 * half;
         a[0] = a[1] = b[0] = b[1] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i0 + row < p.M) {
-            const float* g = (is_v ? p.gV : p.gK) + ((int64_t)u * p.M + i0 + row) * p.d + c0;
+            const float* g = (is_v ? p.gV : p.gK) + ((int64_t)u * p.M + i0 + row) * p.g_st + c0;
             a[0] = load4(g);
             a[1] = load4(g + 4);
         }
@@ -237,13 +259,8 @@ __device__ __forceinline__ void dw_body(const BwdStep& p, float* smem, int block
                 for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(g[x], z[y], acc[x][y]);
         }
     }
-    const int j = j0 + 4 * tj;
-    if (j >= p.S) return;
 #pragma unroll
-    for (int x = 0; x < 8; ++x) {
-        const int i = i0 + (x < 4 ? 4 * ti + x : 32 + 4 * ti + x - 4);
-        if (i < p.M) *reinterpret_cast<float4*>(p.dA + ((int64_t)u * p.M + i) * p.Sr + j) = make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]);
-    }
+    for (int x = 0; x < 8; ++x) out(u, i0 + (x < 4 ? 4 * ti + x : 32 + 4 * ti + x - 4), j0 + 4 * tj, make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]));
 }
 
 template <typename T, int D, int OT>
@@ -264,7 +281,9 @@ __global__ void __launch_bounds__(256) front_kernel(const __grid_constant__ BwdS
     if (x < n_conv2) {
         if (x < n_conv) conv_body<T, OT>(fwd, smem + group * (WindowConv<T, OT>::smem_bytes(p.k) / 4), x, tid, group);
     } else if (x - n_conv2 < n_dw) {
-        dw_body<T>(p, smem + group * kDwFloats, x - n_conv2, tid, group);
+        dw_body<T>(p, smem + group * kDwFloats, x - n_conv2, tid, group, [&](int u, int i, int j, const float4& v) {
+            if (i < p.M && j < p.S) store4(p.dA + ((int64_t)u * p.M + i) * p.Sr + j, v);
+        });
     }
 }
 
@@ -330,64 +349,77 @@ struct SlotRows {      // rows [slot][position] of a unit, scaled row by row whe
     }
 };
 
-template <typename T>
-__device__ __forceinline__ void dx_body(const BwdStep& p, float* parts, int splits, float* smem, int block) {
-    constexpr int PT = 64;
-    const int pos_tiles = (p.S + PT - 1) / PT, ch_tiles = 2 * p.d / 64;
-    const int jt = block % pos_tiles; block /= pos_tiles;
-    const int u = block % p.units; block /= p.units;
-    const int split = block % splits, ct = block / splits;
-    const int h = u % p.heads, pad = (p.k - 1) / 2, j0 = jt * PT, ch0 = ct * 64;
-    const int chunks = (p.M + 7) / 8, c_begin = chunks * split / splits, c_end = chunks * (split + 1) / splits;
-    ConvAcc acc;
+// Positions j0 .. j0 + 63, channels 64 ct .. 64 ct + 63 of [keys | values], slots 8 c_begin .. 8 c_end - 1; `out(j, ch, v)` takes four
+// consecutive channels of row j. kSums: sixteen slots at a time (where the slots are not split over blocks).
+template <typename T, bool kSums, typename Out>
+__device__ __forceinline__ void dx_tile(const BwdStep& p, int u, int j0, int ct, int c_begin, int c_end, float* smem, const Out& out) {
+    const int h = u % p.heads, pad = (p.k - 1) / 2, ch0 = ct * 64;
+    ConvAcc acc, total;
     acc.clear();
+    if (kSums) total.clear();
     if (ch0 < p.c_in) {
         const T* w = reinterpret_cast<const T*>(p.g_reverse) + (p.weights_per_head ? (int64_t)h * p.k * p.M * p.c_in : 0);
         const SlotRows in{p.dA + (int64_t)u * p.M * p.Sr, nullptr, p.M, p.S, p.Sr};
-        WindowConv<T, 64>::run(w, p.M, p.c_in, p.k, ch0, j0 - pad, c_begin, c_end, in, smem, acc, threadIdx.x, 0);
+        WindowConv<T, 64>::template run<kSums>(w, p.M, p.c_in, p.k, ch0, j0 - pad, c_begin, c_end, in, smem, acc, threadIdx.x, 0, &total);
         __syncthreads();
     }
-    const float* g = (ch0 < p.d ? p.gK : p.gV) + (int64_t)u * p.M * p.d;
+    const float* g = (ch0 < p.d ? p.gK : p.gV) + (int64_t)u * p.M * p.g_st;
     const SlotRows in{p.R + (int64_t)u * p.M * p.Sr, p.s + (int64_t)u * p.M, p.M, p.S, p.Sr};
-    WindowConv<float, 64>::run(g, p.M, p.d, 1, ch0 < p.d ? ch0 : ch0 - p.d, j0, c_begin, c_end, in, smem, acc, threadIdx.x, 0);
+    WindowConv<float, 64>::run<kSums>(g, p.M, p.g_st, 1, ch0 < p.d ? ch0 : ch0 - p.d, j0, c_begin, c_end, in, smem, acc, threadIdx.x, 0, &total);
+    const ConvAcc& sum = kSums ? total : acc;
     const int ti = threadIdx.x & 7, tj = threadIdx.x >> 3;
-    float* dst = parts + ((int64_t)split * p.units + u) * p.S * (2 * p.d) + ch0 + 4 * ti;
 #pragma unroll
     for (int y = 0; y < 4; ++y) {
         const int j = j0 + 4 * tj + y;
         if (j >= p.S) break;
-        store4(dst + (int64_t)j * 2 * p.d, make_float4(acc.get(0, y), acc.get(1, y), acc.get(2, y), acc.get(3, y)));
-        store4(dst + (int64_t)j * 2 * p.d + 32, make_float4(acc.get(4, y), acc.get(5, y), acc.get(6, y), acc.get(7, y)));
+        out(j, ch0 + 4 * ti, make_float4(sum.get(0, y), sum.get(1, y), sum.get(2, y), sum.get(3, y)));
+        out(j, ch0 + 4 * ti + 32, make_float4(sum.get(4, y), sum.get(5, y), sum.get(6, y), sum.get(7, y)));
     }
+}
+template <typename T>
+__device__ __forceinline__ void dx_body(const BwdStep& p, float* parts, int splits, float* smem, int block) {
+    const int pos_tiles = (p.S + 63) / 64;
+    const int jt = block % pos_tiles; block /= pos_tiles;
+    const int u = block % p.units; block /= p.units;
+    const int split = block % splits, ct = block / splits;
+    const int chunks = (p.M + 7) / 8;
+    float* dst = parts + ((int64_t)split * p.units + u) * p.S * (2 * p.d);
+    dx_tile<T, false>(p, u, 64 * jt, ct, chunks * split / splits, chunks * (split + 1) / splits, smem,
+                      [&](int j, int ch, const float4& v) { store4(dst + (int64_t)j * 2 * p.d + ch, v); });
 }
 
 // ------------------------------------------------------------------ dG
 // dG[set][i][ch][t] += sum over the set's units, sum_j dA[u][i][j] * Z_u[j+t-pad][ch].
-// A block of 128 threads takes 16 slots x 32 channels x 8 taps and one stretch of positions of one unit: a lane owns a
+// A block of 128 threads takes 16 slots x 32 channels x up to 8 taps and one stretch of positions of one unit: a lane owns a
 // channel, a warp four slots; eight positions at a time, the 15 inputs they and eight taps touch sit in registers and serve
 // 256 FMAs together with eight vector loads of dA. Blocks of the same set meet in atomics.
 constexpr int kGTaps = 8, kGPos = 64, kGSlots = 16;
-template <typename T>
-__device__ __forceinline__ void dg_body(const BwdStep& p, int pieces, float* smem, int block) {
+// Taps per block: at most eight, as few as cover k in as many blocks (kT, what the code is unrolled for: 5 to 8, no fewer).
+__host__ __device__ inline int g_taps(int k) { const int tiles = (k + kGTaps - 1) / kGTaps; return (k + tiles - 1) / tiles; }
+// `stage(q, dA, xk, xv, S, j0)`: the q-th stretch of 64 positions (of all that are to be summed: one chunk's, or several chunks').
+template <typename T, int kT, typename Stage>
+__device__ __forceinline__ void dg_tile(const BwdStep& p, int pieces, int stages, float* smem, int block, const Stage& stage) {
     float* As = smem;                        // [16 slots][64 positions], row stride 68
     float* Zs = smem + kGSlots * 68;         // [64 + 8 positions][32 channels], row stride 33
     const int slot_tiles = (p.M + kGSlots - 1) / kGSlots, ch_tiles = p.c_in / 32;
     const int piece = block % pieces; block /= pieces;
     const int u = block % p.units; block /= p.units;
     const int ch0 = (block % ch_tiles) * 32; block /= ch_tiles;
-    const int i0 = (block % slot_tiles) * kGSlots, t0 = (block / slot_tiles) * kGTaps;
+    const int i0 = (block % slot_tiles) * kGSlots, taps = g_taps(p.k), t0 = (block / slot_tiles) * taps;
     const int n = u / p.heads, h = u % p.heads, set = p.weights_per_head ? h : 0, pad = (p.k - 1) / 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int stages = (p.S + kGPos - 1) / kGPos;
-    const float* dA = p.dA + (int64_t)u * p.M * p.Sr;
-    float acc[4][kGTaps];
+    float acc[4][kT];
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int t = 0; t < kGTaps; ++t) acc[x][t] = 0.f;
+        for (int t = 0; t < kT; ++t) acc[x][t] = 0.f;
 #pragma unroll 1
     for (int st = stages * piece / pieces; st < stages * (piece + 1) / pieces; ++st) {
-        const int j0 = st * kGPos;
+        const float* dA;
+        CatView xk, xv;
+        int S, j0;
+        if (!stage(st, dA, xk, xv, S, j0)) continue;
+        dA += (int64_t)u * p.M * p.Sr;
         __syncthreads();
         for (int x = tid; x < kGSlots * (kGPos / 4); x += 128) {
             const int r = x / (kGPos / 4), q = 4 * (x % (kGPos / 4));
@@ -398,16 +430,16 @@ __device__ __forceinline__ void dg_body(const BwdStep& p, int pieces, float* sme
         for (int x = tid; x < (kGPos + kGTaps) * 8; x += 128) {
             const int r = x >> 3, q = 4 * (x & 7), j = j0 + r + t0 - pad, ch = ch0 + q;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (j >= 0 && j < p.S) v = load4(ch < p.d ? cat_row<T>(p.xk, n, h, j) + ch : cat_row<T>(p.xv, n, h, j) + ch - p.d);
+            if (j >= 0 && j < S) v = load4(ch < p.d ? cat_row<T>(xk, n, h, j) + ch : cat_row<T>(xv, n, h, j) + ch - p.d);
             float* d = Zs + r * 33 + q;
             d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
         }
         __syncthreads();
 #pragma unroll 1
         for (int j = 0; j < kGPos; j += 8) {
-            float z[8 + kGTaps - 1];
+            float z[8 + kT - 1];
 #pragma unroll
-            for (int e = 0; e < 8 + kGTaps - 1; ++e) z[e] = Zs[(j + e) * 33 + lane];
+            for (int e = 0; e < 8 + kT - 1; ++e) z[e] = Zs[(j + e) * 33 + lane];
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
                 const float4 a0 = *reinterpret_cast<const float4*>(As + (4 * warp + x) * 68 + j), a1 = *reinterpret_cast<const float4*>(As + (4 * warp + x) * 68 + j + 4);
@@ -415,7 +447,7 @@ __device__ __forceinline__ void dg_body(const BwdStep& p, int pieces, float* sme
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
 #pragma unroll
-                    for (int t = 0; t < kGTaps; ++t) acc[x][t] = fmaf(a[e], z[e + t], acc[x][t]);
+                    for (int t = 0; t < kT; ++t) acc[x][t] = fmaf(a[e], z[e + t], acc[x][t]);
             }
         }
     }
@@ -425,8 +457,18 @@ __device__ __forceinline__ void dg_body(const BwdStep& p, int pieces, float* sme
         if (i >= p.M) break;
         float* out = p.dG + (((int64_t)set * p.M + i) * p.c_in + ch0 + lane) * p.k + t0;
 #pragma unroll
-        for (int t = 0; t < kGTaps; ++t)
-            if (t0 + t < p.k) atomicAdd(out + t, acc[x][t]);
+        for (int t = 0; t < kT; ++t)
+            if (t < taps && t0 + t < p.k) atomicAdd(out + t, acc[x][t]);
+    }
+}
+
+template <typename T, typename Stage>
+__device__ __forceinline__ void dg_body(const BwdStep& p, int pieces, int stages, float* smem, int block, const Stage& stage) {
+    switch (g_taps(p.k)) {
+        case 8: return dg_tile<T, 8>(p, pieces, stages, smem, block, stage);
+        case 7: return dg_tile<T, 7>(p, pieces, stages, smem, block, stage);
+        case 6: return dg_tile<T, 6>(p, pieces, stages, smem, block, stage);
+        default: return dg_tile<T, 5>(p, pieces, stages, smem, block, stage);
     }
 }
 
@@ -435,7 +477,10 @@ __global__ void __launch_bounds__(128) dx_dg_kernel(const __grid_constant__ BwdS
     extern __shared__ __align__(16) float smem[];
     start_and_wait();
     if ((int)blockIdx.x < n_dx) dx_body<T>(p, parts, splits, smem, blockIdx.x);
-    else dg_body<T>(p, pieces, smem, blockIdx.x - n_dx);
+    else dg_body<T>(p, pieces, (p.S + kGPos - 1) / kGPos, smem, blockIdx.x - n_dx, [&](int q, const float*& dA, CatView& xk, CatView& xv, int& S, int& j0) {
+        dA = p.dA; xk = p.xk; xv = p.xv; S = p.S; j0 = q * kGPos;
+        return true;
+    });
 }
 
 // ------------------------------------------------------------------ split
@@ -522,6 +567,336 @@ int step_typed(const BwdStep& p, CompressParams fwd, float* parts, cudaStream_t 
     return n + 1;
 }
 
+// ------------------------------------------------------------------ groups of chunks
+// Of a step's work only the cache rows' dw, dA and dX wait for the step behind it. For problems of which one chunk does not fill the chip,
+// everything else is done for a whole group of chunks at a time:
+//   group_front   attention gradients (dQ, shares of dX) and the recomputed convolution, all chunks side by side
+//   group_rows    R, s; the cache after the call's last chunk
+//   (simt_chain)  the chain through the cache gradient, one launch for all steps
+//   group_logits  dA (and dbias) at all positions
+//   group_out     dK, dV of the chunks' rows, and dG
+// 8 units, M = 48, B = 100, d = 64, k = 5, 8 chunks: 171 us where the four launches of every step took 380 (front 59, rows 9, chain 36, logits 17, out 49).
+__device__ __forceinline__ void step_of(const BwdGroup& G, int i, BwdStep& p) {
+    p = G.first;
+    const int n = G.n0 + i, t0 = n * G.B;
+    p.c = min(p.M, G.c0 + t0);
+    p.b = min(G.B, G.L - t0);
+    p.S = p.c + p.b;
+    p.Sr = G.Sr;
+    auto tokens = [&](View& v) { v.ptr += (int64_t)t0 * v.st * 4; };
+    tokens(p.xk.chunk); tokens(p.xv.chunk); tokens(p.q); tokens(p.o); tokens(p.d_o); tokens(p.dq); tokens(p.dk); tokens(p.dv);
+    p.xk.cache.ptr += n * G.snap_step * 4;
+    p.xv.cache.ptr += n * G.snap_step * 4;
+    p.xk.c = p.xv.c = p.c;
+    p.xk.b = p.xv.b = p.b;
+    p.lse += t0;
+    p.delta += t0;
+    const int64_t rows = (int64_t)i * p.units * p.M;
+    p.R = G.R + rows * G.splits * G.Sr;
+    p.s = G.s + rows;
+    p.dA = G.dA + rows * G.Sr;
+    p.gK = G.g + (rows + (int64_t)p.units * p.M) * (2 * p.d);        // the gradient w.r.t. the cache after the step
+    p.gV = p.gK + p.d;
+    p.g_st = 2 * p.d;
+}
+__device__ __forceinline__ void logits_of(const BwdGroup& G, const BwdStep& p, CompressParams& f) {
+    f.xk = p.xk; f.xv = p.xv;
+    f.heads = p.heads; f.units = p.units; f.d = p.d; f.M = p.M; f.k = p.k; f.c_in = p.c_in;
+    f.S = p.S; f.Sr = p.Sr; f.splits = G.splits; f.weights_per_head = p.weights_per_head;
+    f.g_packed = G.g_packed; f.bias = G.bias; f.eps = G.eps; f.prot = G.prot; f.R = p.R; f.s = p.s;
+}
+
+template <int D, int OT>
+__global__ void __launch_bounds__(256) group_front_kernel(const __grid_constant__ BwdGroup G, int n_conv) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ BwdStep p;
+    __shared__ __align__(16) unsigned char fwd_bytes[sizeof(CompressParams)];
+    CompressParams& fwd = *reinterpret_cast<CompressParams*>(fwd_bytes);
+    start_and_wait();
+    const int units = G.first.units, each = units * G.count;
+    const int n_keys = (G.S + 31) / 32 * each, n_queries = (G.B + 31) / 32 * each;
+    const int group = threadIdx.x >> 7, tid = threadIdx.x & 127;
+    int x = blockIdx.x;
+    const int kind = x < n_keys ? 0 : (x < n_keys + n_queries ? 1 : 2);
+    x -= kind == 0 ? 0 : (kind == 1 ? n_keys : n_keys + n_queries);
+    const int conv_blocks = (n_conv + 1) / 2;
+    const int i = kind == 2 ? x / conv_blocks : x % each / units;
+    if (threadIdx.x == 0) {
+        step_of(G, i, p);
+        if (kind == 2) logits_of(G, p, fwd);
+    }
+    __syncthreads();
+    if (kind < 2) {
+        // the tiles with the most work first: early keys (every query sees them), late queries
+        const int tile = x / each, u = x % units;
+        if (kind == 0) {
+            if (32 * tile < p.S) attention_grad<float, D, true>(p, G.attn + (int64_t)i * units * G.S * (2 * D), smem, tile, u);
+        } else {
+            const int last = (p.b + 31) / 32 - 1;
+            if (tile <= last) attention_grad<float, D, false>(p, nullptr, smem, last - tile, u);
+        }
+        return;
+    }
+    constexpr int PT = WindowConv<float, OT>::PT;
+    const int tile = 2 * (x % conv_blocks) + group, tiles = (p.S + PT - 1) / PT * ((p.M + OT - 1) / OT) * G.splits * units;
+    if (p.S > p.M && tile < tiles) conv_body<float, OT>(fwd, smem + group * (WindowConv<float, OT>::smem_bytes(p.k) / 4), tile, tid, group);
+}
+
+// R from the partial convolutions and s = sum R + eps, a warp per (chunk, unit, slot); for the last chunk of the call, the first
+// `last_blocks` blocks, also the new cache: a block takes four slots of a unit, two warps each for R, all warps a share of the
+// positions for the blends. (A block per slot read the chunk's rows four times as often: 100 us at 96 units, M = 32, B = 142.)
+__global__ void __launch_bounds__(256) group_rows_kernel(const __grid_constant__ BwdGroup G, int last_blocks) {
+    __shared__ float sums[8];
+    __shared__ __align__(16) float blend[8][4][128];
+    start_and_wait();
+    const int M = G.first.M, rows = G.first.units * M, per_chunk = (rows + 7) / 8, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const bool wide = (int)blockIdx.x < last_blocks;
+    const int x = (int)blockIdx.x - last_blocks, i = wide ? G.count - 1 : x / per_chunk, per_unit = (M + 3) / 4;
+    const int u4 = blockIdx.x / per_unit, i4 = 4 * (blockIdx.x % per_unit), slot4 = min(i4 + warp / 2, M - 1);
+    const int row = wide ? u4 * M + slot4 : x % per_chunk * 8 + warp;
+    BwdStep p;
+    CompressParams fwd;
+    step_of(G, i, p);
+    logits_of(G, p, fwd);
+    if (p.S <= M || row >= rows) return;
+    const LogitRow L(fwd, row);
+    float* R = p.R + (int64_t)row * p.Sr;
+    float sum = 0.f;
+    const bool twice = wide && i4 + warp / 2 >= M;                 // (another pair of warps has this row)
+    for (int j = 4 * (wide ? lane + 32 * (warp & 1) : lane); j < p.Sr && !twice; j += wide ? 256 : 128) {
+        const float4 r = L.at4(j);
+        store4(R + j, r);
+        sum += (r.x + r.y) + (r.z + r.w);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (!wide) {
+        if (lane == 0) p.s[row] = row % M < G.prot ? 1.f : sum + G.eps;
+        return;
+    }
+    if (lane == 0) sums[warp] = sum;
+    __syncthreads();
+    const int n = u4 / p.heads, h = u4 % p.heads;
+    const float* rows4[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) rows4[a] = p.R + (int64_t)(u4 * M + min(i4 + a, M - 1)) * p.Sr;
+#pragma unroll 1
+    for (int ch0 = 0; ch0 < 2 * p.d; ch0 += 128) {
+        const int ch = ch0 + 4 * lane;
+        float4 acc[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) acc[a] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int j = warp; j < p.S; j += 8) {
+            const float4 v = load4(ch < p.d ? cat_row<float>(p.xk, n, h, j) + ch : cat_row<float>(p.xv, n, h, j) + ch - p.d);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) axpy4(rows4[a][j], v, acc[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) store4(&blend[warp][a][4 * lane], acc[a]);
+        __syncthreads();
+        for (int e = threadIdx.x; e < 512; e += 256) {
+            const int a = e / 128, c = e % 128, slot = i4 + a;
+            if (slot >= M || ch0 + c >= 2 * p.d) continue;
+            float v[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) v[w] = blend[2 * w][a][c] + blend[2 * w + 1][a][c];
+            const float s = slot < G.prot ? 1.f : sums[2 * a] + sums[2 * a + 1] + G.eps;
+            if (ch0 + c == 0) p.s[u4 * M + slot] = s;
+            G.last[((int64_t)u4 * M + slot) * (2 * p.d) + ch0 + c] = ((v[0] + v[1]) + (v[2] + v[3])) * (1.f / s);
+        }
+        __syncthreads();
+    }
+}
+
+// dw at all positions, and dA: a block of 256 threads takes 16 or 32 slots (32 where that leaves fewer than 16 idle: the rows are then
+// read half as often) x 128 positions of a unit, 2 or 4 x 4 per thread; keys and values with their
+// gradients come whole (asynchronous copies, the values while the keys' half is summed). (With 64 x 64 tiles by groups of 128
+// threads, sixteen channels per barrier: 32 us at 8 units, M = 48, B = 100, 8 chunks; now 17.)
+template <int D, int kSlots>
+struct DwSmem {
+    static constexpr int kRow = D + 4, kRows = 128 + kSlots, kHalf = kRows * kRow, kFloats = 2 * kHalf;
+};
+template <int D, int kSlots>
+__global__ void __launch_bounds__(256) group_logits_kernel(const __grid_constant__ BwdGroup G) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ float bias_part[8][kSlots];
+    start_and_wait();
+    using Smem = DwSmem<D, kSlots>;
+    constexpr int RS = Smem::kRow, kA = kSlots / 8;      // slots per thread: ti, ti + 8, ...
+    const int tid = threadIdx.x, lane = tid & 31, ti = tid & 7, tj = tid >> 3;
+    const int pos_tiles = (G.S + 127) / 128, slot_tiles = (G.first.M + kSlots - 1) / kSlots;
+    int x = blockIdx.x;
+    const int j0 = 128 * (x % pos_tiles); x /= pos_tiles;
+    const int i0 = kSlots * (x % slot_tiles); x /= slot_tiles;
+    const int u = x % G.first.units, i = x / G.first.units;
+    BwdStep p;
+    step_of(G, i, p);
+    if (p.S <= p.M || j0 >= p.S) return;
+    const int n = u / p.heads, h = u % p.heads;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        const CatView& xs = half ? p.xv : p.xk;
+        const float *cache = unit_base<float>(xs.cache, n, h), *chunk = unit_base<float>(xs.chunk, n, h);
+        const float* g = (half ? p.gV : p.gK) + ((int64_t)u * p.M + i0) * p.g_st;
+        float* dst = smem + half * Smem::kHalf;
+        const int ch = 4 * (tid % (D / 4));
+        for (int r = tid / (D / 4); r < Smem::kRows; r += 256 / (D / 4)) {
+            const int j = j0 + r;
+            const bool live = r < 128 ? j < p.S : i0 + r - 128 < p.M;
+            const float* src = r >= 128 ? g + (int64_t)(r - 128) * p.g_st : (j < p.c ? cache + (int64_t)j * xs.cache.st : chunk + (int64_t)(j - p.c) * xs.chunk.st);
+            cp_async16(dst + r * RS + ch, live ? src + ch : cache, live);
+        }
+        cp_async_commit();
+    }
+    f32x2 acc[kA][4];
+#pragma unroll
+    for (int a = 0; a < kA; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0ull;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        if (half) cp_async_wait<0>();
+        else cp_async_wait<1>();
+        __syncthreads();
+        const float *xr = smem + half * Smem::kHalf + tj * RS, *gr = smem + half * Smem::kHalf + (128 + ti) * RS;
+#pragma unroll 2
+        for (int q = 0; q < D / 4; ++q) {
+            f32x4 z[4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) z[b] = load_pairs(xr + 32 * b * RS + 4 * q);
+#pragma unroll
+            for (int a = 0; a < kA; ++a) {
+                const f32x4 w = load_pairs(gr + 8 * a * RS + 4 * q);
+#pragma unroll
+                for (int b = 0; b < 4; ++b) { fma2(w.lo, z[b].lo, acc[a][b]); fma2(w.hi, z[b].hi, acc[a][b]); }
+            }
+        }
+    }
+    const float* inner = G.inner + ((int64_t)i * p.units + u) * p.M;
+#pragma unroll
+    for (int a = 0; a < kA; ++a) {
+        const int slot = i0 + ti + 8 * a, row = u * p.M + slot;
+        float sum = 0.f;
+        if (slot < p.M) {
+            const float inv = 1.f / p.s[row], in = inner[slot];
+            const float* R = p.R + (int64_t)row * p.Sr;
+            float* dA = p.dA + (int64_t)row * p.Sr;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int j = j0 + tj + 32 * b;
+                if (j >= p.Sr) break;
+                const float2 f = unpair(acc[a][b]);
+                const float v = slot >= G.prot && R[j] > 0.f ? (f.x + f.y - in) * inv : 0.f;      // (a protected slot's row has no gradient)
+                dA[j] = v;
+                sum += v;
+            }
+        }
+        if (p.dbias) {                                   // lanes ti, ti + 8, ... hold positions of the same slot
+#pragma unroll
+            for (int o = 8; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane < 8) bias_part[tid >> 5][ti + 8 * a] = sum;
+        }
+    }
+    if (!p.dbias) return;
+    __syncthreads();
+    if (tid < kSlots && i0 + tid < p.M) {
+        float v[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) v[w] = bias_part[2 * w][tid] + bias_part[2 * w + 1][tid];
+        atomicAdd(p.dbias + (p.weights_per_head ? h * p.M : 0) + i0 + tid, (v[0] + v[1]) + (v[2] + v[3]));
+    }
+}
+
+__global__ void __launch_bounds__(128) group_out_kernel(const __grid_constant__ BwdGroup G, int n_dx, int pieces) {
+    extern __shared__ __align__(16) float smem[];
+    start_and_wait();
+    const BwdStep& F = G.first;
+    int x = blockIdx.x;
+    if (x >= n_dx) {
+        const int per = (G.S + kGPos - 1) / kGPos;
+        dg_body<float>(F, pieces, per * G.count, smem, x - n_dx, [&](int q, const float*& dA, CatView& xk, CatView& xv, int& S, int& j0) {
+            const int i = q / per, n = G.n0 + i, t0 = n * G.B, c = min(F.M, G.c0 + t0);
+            j0 = (q - i * per) * kGPos;
+            S = c + min(G.B, G.L - t0);
+            if (S <= F.M || j0 >= S) return false;
+            dA = G.dA + (int64_t)i * F.units * F.M * G.Sr;
+            xk = F.xk; xv = F.xv;
+            xk.cache.ptr += n * G.snap_step * 4; xv.cache.ptr += n * G.snap_step * 4;
+            xk.chunk.ptr += (int64_t)t0 * xk.chunk.st * 4; xv.chunk.ptr += (int64_t)t0 * xv.chunk.st * 4;
+            xk.c = xv.c = c;
+            return true;
+        });
+        return;
+    }
+    const int tiles = (G.B + 63) / 64, jt = x % tiles; x /= tiles;
+    const int ct = x % (F.d / 32); x /= F.d / 32;
+    const int u = x % F.units, i = x / F.units;
+    BwdStep p;
+    step_of(G, i, p);
+    if (64 * jt >= p.b) return;
+    const int n = u / p.heads, h = u % p.heads;
+    const float* attn = G.attn + ((int64_t)i * p.units * G.S + (int64_t)u * p.S) * (2 * p.d);
+    auto put = [&](int j, int ch, const float4& v) {
+        const bool is_v = ch >= p.d;
+        const View& out = is_v ? p.dv : p.dk;
+        const float4 a = load4(attn + (int64_t)j * (2 * p.d) + ch);
+        store4(unit_base_mut<float>(out, n, h) + (int64_t)(j - p.c) * out.st + (is_v ? ch - p.d : ch), make_float4(v.x + a.x, v.y + a.y, v.z + a.z, v.w + a.w));
+    };
+    const int j0 = p.c + 64 * jt;
+    if (p.S > p.M) {
+        dx_tile<float, true>(p, u, j0, ct, 0, (p.M + 7) / 8, smem, put);
+        return;
+    }
+    // a fill step: the gradient of the filled cache itself
+    for (int e = threadIdx.x; e < 64 * 16; e += 128) {
+        const int j = j0 + e / 16, ch = 64 * ct + 4 * (e % 16);
+        if (j < p.S) put(j, ch, load4(p.gK + ((int64_t)u * p.M + j) * p.g_st + ch));
+    }
+}
+
+template <int D, int OT>
+int launch_group_front(const BwdGroup& G, cudaStream_t st) {
+    static bool done[64] = {};
+    if (!smem_limit(group_front_kernel<D, OT>, 200 * 1024, done)) return -1;
+    const int each = G.first.units * G.count, pt = WindowConv<float, OT>::PT;
+    const int n_conv = (G.S + pt - 1) / pt * ((G.first.M + OT - 1) / OT) * G.splits * G.first.units;
+    const size_t smem = std::max(sizeof(float) * (size_t)GradSmem<D>::kFloats, 2 * WindowConv<float, OT>::smem_bytes(G.first.k));
+    const int64_t blocks = (int64_t)((G.S + 31) / 32 + (G.B + 31) / 32) * each + (int64_t)(n_conv + 1) / 2 * G.count;
+    return launch_after(group_front_kernel<D, OT>, dim3((unsigned)blocks), dim3(256), smem, st, G, n_conv) ? 1 : -1;
+}
+template <int D>
+int launch_group_front_tiles(const BwdGroup& G, cudaStream_t st) {
+    switch (slot_tile(G.first.M)) {
+        case 64: return launch_group_front<D, 64>(G, st);
+        case 32: return launch_group_front<D, 32>(G, st);
+        default: return launch_group_front<D, 16>(G, st);
+    }
+}
+
+template <int D, int kSlots>
+int launch_group_logits(const BwdGroup& G, cudaStream_t st) {
+    static bool done[64] = {};
+    const int smem = sizeof(float) * DwSmem<D, kSlots>::kFloats, blocks = (G.S + 127) / 128 * ((G.first.M + kSlots - 1) / kSlots) * G.first.units * G.count;
+    if (!smem_limit(group_logits_kernel<D, kSlots>, smem, done)) return -1;
+    return launch_after(group_logits_kernel<D, kSlots>, dim3(blocks), dim3(256), smem, st, G) ? 1 : -1;
+}
+template <int D>
+int launch_group_logits_tiles(const BwdGroup& G, cudaStream_t st) {
+    return (G.first.M + 31) / 32 * 32 - G.first.M < 16 ? launch_group_logits<D, 32>(G, st) : launch_group_logits<D, 16>(G, st);
+}
+
+// Partial sums per tile of the recomputed convolution, as in conv_splits, for the tiles of all chunks together.
+int group_splits(int units, int M, int S, int c_in, int chunks) {
+    const int OT = slot_tile(M), PT = 4096 / OT;
+    const int64_t tiles = (int64_t)((S + PT - 1) / PT) * ((M + OT - 1) / OT) * units * chunks;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(6 * kSMs / tiles, c_in / 32));
+}
+size_t group_floats(int units, int M, int S, int d, int c_in, int chunks) {
+    const size_t rows = (size_t)units * M, Sr = (S + 3) / 4 * 4;
+    return chunks * ((size_t)units * S * 2 * d + rows * Sr * (group_splits(units, M, S, c_in, chunks) + 1) + 2 * ((rows + 3) / 4 * 4)) + (chunks + 2) * rows * 2 * d;
+}
+
 }  // namespace
 
 size_t simt_backward_parts_floats(int units, int M, int B, int d) {
@@ -539,6 +914,56 @@ int simt_backward_fill_split(int dtype, const BwdStep& p, const float* attn, cud
 
 int simt_backward_step(int dtype, const BwdStep& p, const CompressParams& fwd, float* parts, cudaStream_t st) {
     return dtype == LOCOCO_F32 ? step_typed<float>(p, fwd, parts, st) : step_typed<__nv_bfloat16>(p, fwd, parts, st);
+}
+
+int simt_group_chunks(const lococo_handle* h, int L, int B, size_t* floats) {
+    const lococo_config& c = h->cfg;
+    B = std::min(B, L);
+    const int chunks = (L + B - 1) / B;
+    if (c.dtype != LOCOCO_F32 || chunks < 2 || (size_t)c.M * c.head_dim > 6144) return 0;      // (larger caches: not in simt_chain.cu's shared memory)
+    // Where the attention's blocks of one chunk alone are more than six per SM, single steps are as fast and take less memory (96 units,
+    // M = 32, B = 142: 571 us a step at a time, 588 in one group; 112 units of d = 128, M = 16, B = 77, 672 blocks per chunk: 1013 / 823).
+    if ((int64_t)((c.M + B + 31) / 32 + (B + 31) / 32) * h->units > 6 * kSMs) return 0;
+    // as many chunks as 128 MB hold
+    int n = std::min(chunks, 4096);
+    while (n > 1 && group_floats(h->units, c.M, c.M + B, c.head_dim, c.c_in, n) > (32u << 20)) n = std::min(n - 1, (n * 7 + 7) / 8);
+    if (n < 2) return 0;
+    *floats = group_floats(h->units, c.M, c.M + B, c.head_dim, c.c_in, n);
+    return n;
+}
+
+void simt_group_layout(BwdGroup& G, float* at) {
+    const BwdStep& p = G.first;
+    const size_t rows = (size_t)p.units * p.M;
+    G.splits = group_splits(p.units, p.M, G.S, p.c_in, G.count);
+    auto take = [&](size_t floats) { float* r = at; at += floats; return r; };
+    G.attn = take((size_t)G.count * p.units * G.S * 2 * p.d);
+    G.R = take(G.count * rows * G.Sr * G.splits);
+    G.dA = take(G.count * rows * G.Sr);
+    G.g = take((G.count + 1) * rows * 2 * p.d);
+    G.last = take(rows * 2 * p.d);
+    G.s = take(G.count * ((rows + 3) / 4 * 4));
+    G.inner = take(G.count * ((rows + 3) / 4 * 4));
+}
+
+int simt_backward_group(const BwdGroup& G, cudaStream_t st) {
+    const BwdStep& p = G.first;
+    const int rows = p.units * p.M;
+    static bool done[64] = {};
+    if ((p.d == 128 ? launch_group_front_tiles<128>(G, st) : launch_group_front_tiles<64>(G, st)) < 0) return -1;
+    const int last = (G.n0 + G.count) * (int64_t)G.B >= G.L, last_blocks = last ? (p.M + 3) / 4 * p.units : 0;
+    if (!launch_after(group_rows_kernel, dim3(last_blocks + (rows + 7) / 8 * (G.count - last)), dim3(256), 0, st, G, last_blocks)) return -1;
+    if (simt_backward_chain(G, st) < 0) return -1;
+    if ((p.d == 128 ? launch_group_logits_tiles<128>(G, st) : launch_group_logits_tiles<64>(G, st)) < 0) return -1;
+    const int n_dx = (G.B + 63) / 64 * (p.d / 32) * p.units * G.count;
+    // dG: stretches of the group's positions per unit, so that about six blocks per SM exist, none shorter than a stage
+    const int tiles = (p.k + kGTaps - 1) / kGTaps * ((p.M + kGSlots - 1) / kGSlots) * (p.c_in / 32) * p.units;
+    const int stages = (G.S + kGPos - 1) / kGPos * G.count, most = std::max(1, std::min(stages, 6 * kSMs / std::max(1, tiles)));
+    const int pieces = (stages + (stages + most - 1) / most - 1) / ((stages + most - 1) / most);      // (as many stages each)
+    const size_t smem = std::max(WindowConv<float, 64>::smem_bytes(p.k), sizeof(float) * (kGSlots * 68 + (kGPos + kGTaps) * 33));
+    if (!smem_limit(group_out_kernel, 64 * 1024, done)) return -1;
+    if (!launch_after(group_out_kernel, dim3(n_dx + tiles * pieces), dim3(128), smem, st, G, n_dx, pieces)) return -1;
+    return 5;
 }
 
 }  // namespace lococo

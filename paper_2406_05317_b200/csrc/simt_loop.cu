@@ -77,28 +77,6 @@ __host__ __device__ inline LoopLayout loop_layout(int d, int M, int B, int k, in
     return l;
 }
 
-// Sums of v[0..N-1] over the L lanes of a group (powers of two); lane l of the group is left with max(1, N / L) results in
-// v[0..], from index l * N / L on (L > N: every L / N lanes hold the same one).
-template <int N, int L>
-__device__ __forceinline__ void reduce_lanes(float (&v)[N], int lane) {
-    int n = N;
-#pragma unroll
-    for (int m = L / 2; m > 0; m >>= 1) {
-        if (n == 1) {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
-            continue;
-        }
-        n >>= 1;
-        const bool up = lane & m;
-#pragma unroll
-        for (int e = 0; e < N / 2; ++e) {
-            if (e >= n) break;
-            const float send = up ? v[e] : v[e + n], keep = up ? v[e + n] : v[e];
-            v[e] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-        }
-    }
-}
-
 // One row of a tile of dot products: acc[b] += over this lane's four channels x . y[(b + first) % NB]
 template <int NB>
 __device__ __forceinline__ void row_fma(const f32x4& x, const f32x4 (&y)[NB], int first, f32x2* acc) {
