@@ -165,6 +165,7 @@ __device__ __forceinline__ float2 unpair(f32x2 v) {
     return r;
 }
 __device__ __forceinline__ void fma2(f32x2 a, f32x2 b, f32x2& acc) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b)); }
+__device__ __forceinline__ void add2(f32x2 a, f32x2& acc) { asm("add.rn.f32x2 %0, %1, %0;" : "+l"(acc) : "l"(a)); }
 __device__ __forceinline__ void mul2(f32x2 a, f32x2& acc) { asm("mul.rn.f32x2 %0, %1, %0;" : "+l"(acc) : "l"(a)); }
 struct f32x4 { f32x2 lo, hi; };                  // a float4 as two operands
 __device__ __forceinline__ f32x4 load_pairs(const float* p) {
