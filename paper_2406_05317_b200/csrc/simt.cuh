@@ -51,6 +51,12 @@ __device__ __forceinline__ void start_and_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// Kernels with long blocks let the next launch in only when their blocks end. Blocks that wait are placed where room is first, two on an SM that
+// is done early while others get none, and stay there: that costs more than a launch that is not hidden. Triggered at the start of
+// blends, convolutions and the backward launches -> at their end: 12 heads of 128, 5 chunks of 200, M = 128, k = 21 759 -> 715 us, 3 heads 464 -> 341;
+// k = 5 and 8 heads, 4 of 512 496 -> 449; a training step of 8 heads, 4 of 300, k = 21 3446 -> 3126. Worst of 76 sizes: 16 heads, k = 13 892 -> 900.
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (`overlap` false: in plain stream order.)
 template <typename... Params, typename... Args>
 inline bool launch_maybe_after(bool overlap, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {

@@ -266,7 +266,7 @@ __device__ __forceinline__ void dw_body(const BwdStep& p, float* smem, int block
 template <typename T, int D, int OT>
 __global__ void __launch_bounds__(256) front_kernel(const __grid_constant__ BwdStep p, const __grid_constant__ CompressParams fwd, float* dx_attn, int n_attn, int n_conv, int n_dw) {
     extern __shared__ __align__(16) float smem[];
-    start_and_wait();
+    wait_for_previous();
     const int key_tiles = (p.S + 31) / 32, n_keys = key_tiles * p.units;
     const int group = threadIdx.x >> 7, tid = threadIdx.x & 127;
     int x = blockIdx.x;
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(256) front_kernel(const __grid_constant__ BwdS
 // One warp per (unit, slot) row: R from the partial convolutions, s = sum R + eps, inner = <dw, R>/s;
 // dA = [R>0] (dw - inner)/s;  dbias += sum_j dA. (Columns from S on are zeros in R and in dA.)
 __global__ void __launch_bounds__(256) rows_kernel(const __grid_constant__ BwdStep p, const __grid_constant__ CompressParams fwd) {
-    start_and_wait();
+    wait_for_previous();
     const int row = blockIdx.x * 8 + threadIdx.x / 32;
     if (row >= p.units * p.M) return;
     const int lane = threadIdx.x % 32;
@@ -475,7 +475,7 @@ __device__ __forceinline__ void dg_body(const BwdStep& p, int pieces, int stages
 template <typename T>
 __global__ void __launch_bounds__(128) dx_dg_kernel(const __grid_constant__ BwdStep p, float* parts, int splits, int n_dx, int pieces) {
     extern __shared__ __align__(16) float smem[];
-    start_and_wait();
+    wait_for_previous();
     if ((int)blockIdx.x < n_dx) dx_body<T>(p, parts, splits, smem, blockIdx.x);
     else dg_body<T>(p, pieces, (p.S + kGPos - 1) / kGPos, smem, blockIdx.x - n_dx, [&](int q, const float*& dA, CatView& xk, CatView& xv, int& S, int& j0) {
         dA = p.dA; xk = p.xk; xv = p.xv; S = p.S; j0 = q * kGPos;
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(128) dx_dg_kernel(const __grid_constant__ BwdS
 // the gradient w.r.t. the cache before this step (rows >= c: zero); rows c..S-1 are this chunk's dK, dV.
 template <typename T>
 __global__ void __launch_bounds__(256) split_kernel(const __grid_constant__ BwdStep p, const float* attn, const float* parts, int n_parts) {
-    start_and_wait();
+    wait_for_previous();
     const int u = blockIdx.y, n = u / p.heads, h = u % p.heads;
     const int per_row = p.d / 2, rows = max(p.M, p.S);           // float4 pieces of a [key | value] row
     const int64_t step = (int64_t)p.units * p.S * (2 * p.d);
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(256) group_front_kernel(const __grid_constant_
     __shared__ BwdStep p;
     __shared__ __align__(16) unsigned char fwd_bytes[sizeof(CompressParams)];
     CompressParams& fwd = *reinterpret_cast<CompressParams*>(fwd_bytes);
-    start_and_wait();
+    wait_for_previous();
     const int units = G.first.units, each = units * G.count;
     const int n_keys = (G.S + 31) / 32 * each, n_queries = (G.B + 31) / 32 * each;
     const int group = threadIdx.x >> 7, tid = threadIdx.x & 127;
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(256) group_front_kernel(const __grid_constant_
 __global__ void __launch_bounds__(256) group_rows_kernel(const __grid_constant__ BwdGroup G, int last_blocks) {
     __shared__ float sums[8];
     __shared__ __align__(16) float blend[8][4][128];
-    start_and_wait();
+    wait_for_previous();
     const int M = G.first.M, rows = G.first.units * M, per_chunk = (rows + 7) / 8, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const bool wide = (int)blockIdx.x < last_blocks;
     const int x = (int)blockIdx.x - last_blocks, i = wide ? G.count - 1 : x / per_chunk, per_unit = (M + 3) / 4;
@@ -721,7 +721,7 @@ template <int D, int kSlots>
 __global__ void __launch_bounds__(256) group_logits_kernel(const __grid_constant__ BwdGroup G) {
     extern __shared__ __align__(16) float smem[];
     __shared__ float bias_part[8][kSlots];
-    start_and_wait();
+    wait_for_previous();
     using Smem = DwSmem<D, kSlots>;
     constexpr int RS = Smem::kRow, kA = kSlots / 8;      // slots per thread: ti, ti + 8, ...
     const int tid = threadIdx.x, lane = tid & 31, ti = tid & 7, tj = tid >> 3;
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(256) group_logits_kernel(const __grid_constant
 
 __global__ void __launch_bounds__(128) group_out_kernel(const __grid_constant__ BwdGroup G, int n_dx, int pieces) {
     extern __shared__ __align__(16) float smem[];
-    start_and_wait();
+    wait_for_previous();
     const BwdStep& F = G.first;
     int x = blockIdx.x;
     if (x >= n_dx) {

@@ -251,7 +251,8 @@ struct StepParams {
 template <typename T, int D, int OT>
 __global__ void __launch_bounds__(256, 2) step_kernel(const __grid_constant__ StepParams P) {
     extern __shared__ __align__(16) float smem[];
-    start_and_wait();
+    if ((int)blockIdx.x < P.n_attn) start_next();         // (the blends take their places once the convolution's blocks are gone)
+    wait_for_previous();
     if ((int)blockIdx.x < P.n_attn) {
         const int qtiles = (P.a.b + 31) / 32;
         attention_body<T, D>(P.a, smem, qtiles - 1 - (int)blockIdx.x / P.a.units, blockIdx.x % P.a.units);
@@ -282,7 +283,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(256) blend_kernel(CompressParams p, int to_cache) {
     __shared__ __align__(16) float Xs[4][16][64];
     __shared__ __align__(16) float Rs[4][16][16];      // [group][position][slot]
-    start_and_wait();
+    wait_for_previous();
     const int u = blockIdx.z, n = u / p.heads, h = u % p.heads;
     const int i0 = blockIdx.x * 16, cb = blockIdx.y * 64;
     const bool is_v = cb >= D;
