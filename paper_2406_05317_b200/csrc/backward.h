@@ -60,7 +60,7 @@ struct BwdGroup {
 int simt_group_chunks(const lococo_handle* h, int L, int B, size_t* floats);
 // Lays the arrays of G out from `scratch`, which has the room for groups of G.count chunks.
 void simt_group_layout(BwdGroup& G, float* scratch);
-bool simt_group_supported(const BwdGroup& G);      // (clusters of CTAs that this device can run)
+bool simt_group_supported(const BwdGroup& G);      // (clusters of CTAs that this device can run, and not one after another)
 int simt_backward_group(const BwdGroup& G, cudaStream_t st);
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st);      // (simt_chain.cu: the part of a group that is a chain)
 

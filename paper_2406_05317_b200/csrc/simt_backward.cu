@@ -922,7 +922,7 @@ int simt_group_chunks(const lococo_handle* h, int L, int B, size_t* floats) {
     const int chunks = (L + B - 1) / B;
     if (c.dtype != LOCOCO_F32 || chunks < 2 || (size_t)c.M * c.head_dim > 6144) return 0;      // (larger caches: not in simt_chain.cu's shared memory)
     // Where the attention's blocks of one chunk alone are more than six per SM, single steps are as fast and take less memory (96 units,
-    // M = 32, B = 142: 571 us a step at a time, 588 in one group; 112 units of d = 128, M = 16, B = 77, 672 blocks per chunk: 1013 / 823).
+    // M = 32, B = 142: 571 us a step at a time, 588 in one group). simt_group_supported draws a narrower line, by what the device runs at once.
     if ((int64_t)((c.M + B + 31) / 32 + (B + 31) / 32) * h->units > 6 * kSMs) return 0;
     // as many chunks as 128 MB hold
     int n = std::min(chunks, 4096);

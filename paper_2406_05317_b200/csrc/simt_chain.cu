@@ -285,28 +285,38 @@ ClusterKernel chain_state[2];
 template <int D>
 int resident(int ctas) { return resident_clusters(chain_state[D == 128], chain_kernel<D>, kMaxSmem, ctas, kThreads); }
 
-// CTAs per unit: fewest estimated microseconds per step (0: none fits)
-int chain_ctas(const BwdGroup& G) {
+// CTAs per unit (0: none fits) by the fewest estimated microseconds per step, and how many of these are not the step's work spread over all SMs
+struct ChainPlan { int ctas; double us, idle_us; };
+ChainPlan chain_plan(const BwdGroup& G) {
     const BwdStep& p = G.first;
-    int best = 0;
-    double least = 1e30;
+    ChainPlan best{0, 1e30, 0};
     for (int ctas = 1; ctas <= std::min(kMaxCluster, p.M); ctas = ctas < 8 ? 2 * ctas : ctas + 1) {
         const ChainLayout lay = chain_layout(p.d, p.M, p.k, p.c_in, ctas);
         if ((double)lay.slots * p.k * p.c_in * 4 > kMaxSmem || (size_t)lay.total * 4 > kMaxSmem) continue;
         const int clusters = p.d == 128 ? resident<128>(ctas) : resident<64>(ctas);
         if (clusters == 0) continue;
-        const double t = (p.units + clusters - 1) / clusters * (2.0 + 0.03 * ctas + (double)lay.slots * p.M * (4.0 * p.d + (double)p.c_in * p.k) / 90e3);
-        if (t < least) { least = t; best = ctas; }
+        const double per_slot = (double)p.M * (4.0 * p.d + (double)p.c_in * p.k) / 90e3;
+        const double us = (p.units + clusters - 1) / clusters * (2.0 + 0.03 * ctas + lay.slots * per_slot);
+        if (us < best.us) best = {ctas, us, us - per_slot * p.M * p.units / kSMs};
     }
     return best;
 }
 
 }  // namespace
 
-bool simt_group_supported(const BwdGroup& G) { return chain_ctas(G) > 0; }
+// What a group saves is the latency of a step's four launches, about 28 us; what it costs is the chip's time while units wait for others' clusters or
+// for one another's rows, and the attention's blocks (per SM) no longer hide anything where they alone fill the chip. The weights are a
+// least-squares fit to 78 sizes (6 us per step off). d = 128, B = 100, a training step in groups / a step at a time, us: 32 units, M = 32, k = 5
+// 560 / 643; 96, M = 16 1029 / 1047; 24, M = 32, k = 11 612 / 667, 48 1083 / 984; 16, M = 48, k = 5 497 / 527, 32 830 / 781, 96 2178 / 1706.
+bool simt_group_supported(const BwdGroup& G) {
+    const BwdStep& p = G.first;
+    const ChainPlan plan = chain_plan(G);
+    const int attention_blocks = ((p.M + G.B + 31) / 32 + (G.B + 31) / 32) * p.units;
+    return plan.ctas > 0 && 1.9 * plan.idle_us + 4.6 * attention_blocks / kSMs * p.d / 128 <= 28.0;
+}
 
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st) {
-    ChainParams P{G, chain_ctas(G)};
+    ChainParams P{G, chain_plan(G).ctas};
     if (P.ctas == 0) return -1;
     const BwdStep& p = G.first;
     const size_t smem = (size_t)chain_layout(p.d, p.M, p.k, p.c_in, P.ctas).total * 4;

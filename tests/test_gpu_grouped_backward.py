@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
     (1, 2, 64, 40, 20, 130, 63, 1, True, False),      # padding wider than a chunk: the first compress step ends inside it
     (1, 2, 128, 20, 7, 45, 9, 2, False, True),        # two fill steps, then a partly filled cache
     (5, 32, 64, 16, 16, 50, 5, 1, False, False),      # more units than SMs: a CTA per unit
-    (1, 16, 128, 48, 512, 5632, 3, 1, False, True),   # more than one group of chunks
+    (1, 16, 128, 48, 512, 5632, 3, 1, False, True),   # a group's sizes, but its units would wait for one another: a step at a time
+    (1, 8, 128, 48, 512, 10752, 3, 1, False, True),   # more than one group of chunks
     (1, 1, 64, 2, 300, 700, 1, 1, True, True),        # one tap, two slots, a first step without cache and padding
 ])
 def test_grouped_backward(batch, heads, d, M, B, L, k, c_mult, per_head, bias):
