@@ -108,6 +108,7 @@ View bdev(const lococo_tensor& t, int64_t tokens, size_t elt) {
 
 struct Scratch {
     size_t gK, gV, parts, dA, delta, tensor, group, total;
+    size_t group_floats;       // room of the groups
     int group_chunks;          // chunks that one go of the CUDA cores can take (0: a step at a time)
 };
 
@@ -126,10 +127,9 @@ Scratch scratch_layout(const lococo_handle* h, int L, int B) {
         s.parts = take(simt_backward_parts_floats(h->units, c.M, B, c.head_dim) * sizeof(float));
         s.dA = take(units * c.M * ((Smax + 3) / 4 * 4) * sizeof(float));
         // (in the place of what single steps need: a call takes the one way or the other)
-        size_t floats = 0;
         s.group = s.parts;
-        s.group_chunks = simt_group_chunks(h, L, B, &floats);
-        off = std::max(off, s.group + align256(floats * sizeof(float)));
+        s.group_chunks = simt_group_chunks(h, L, B, &s.group_floats);
+        off = std::max(off, s.group + align256(s.group_floats * sizeof(float)));
     }
     s.total = off;
     return s;
@@ -210,6 +210,14 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
         G.gK = gK; G.gV = gV;
     }
     const bool grouped = sl.group_chunks && simt_group_supported(G);
+    // groups n0, n0 + group_chunks, ... from the last chunk back; the one that is left at the front may be shorter
+    auto group_before = [&](int n) {
+        G.count = std::min(n, sl.group_chunks);
+        G.n0 = n - G.count;
+        return simt_group_layout(G, reinterpret_cast<float*>(sc + sl.group), sl.group_floats) <= sl.group_floats;
+    };
+    for (int n = n_chunks; grouped && n > 0; n -= G.count)
+        if (!group_before(n)) return LOCOCO_ERR_WORKSPACE;
     char* tb = tensor_backward_supported(h) ? sc + sl.tensor : nullptr;
     if (tb) {
         const int r = tensor_backward_prepare(h, B, tb, st);
@@ -239,9 +247,7 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
         c = c + b <= cfg.M ? c + b : cfg.M;
     }
     for (int n = n_chunks; grouped && n > 0; n -= G.count) {
-        G.count = std::min(n, sl.group_chunks);
-        G.n0 = n - G.count;
-        simt_group_layout(G, reinterpret_cast<float*>(sc + sl.group));
+        group_before(n);
         const int r = simt_backward_group(G, st);
         if (r < 0) return LOCOCO_ERR_CUDA;
         h->launches += r;

@@ -58,8 +58,8 @@ struct BwdGroup {
 };
 // Chunks of a group (0: one step at a time is the way), and the floats of scratch that a group takes; both depend on the sizes alone.
 int simt_group_chunks(const lococo_handle* h, int L, int B, size_t* floats);
-// Lays the arrays of G out from `scratch`, which has the room for groups of G.count chunks.
-void simt_group_layout(BwdGroup& G, float* scratch);
+// Lays the arrays of G out in the `floats` at `scratch` (what simt_group_chunks said, or less chunks' worth of it), and says how many they take.
+size_t simt_group_layout(BwdGroup& G, float* scratch, size_t floats);
 bool simt_group_supported(const BwdGroup& G);      // (clusters of CTAs that this device can run, and not one after another)
 int simt_backward_group(const BwdGroup& G, cudaStream_t st);
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st);      // (simt_chain.cu: the part of a group that is a chain)

@@ -892,9 +892,9 @@ int group_splits(int units, int M, int S, int c_in, int chunks) {
     const int64_t tiles = (int64_t)((S + PT - 1) / PT) * ((M + OT - 1) / OT) * units * chunks;
     return (int)std::max<int64_t>(1, std::min<int64_t>(6 * kSMs / tiles, c_in / 32));
 }
-size_t group_floats(int units, int M, int S, int d, int c_in, int chunks) {
+size_t group_floats(int units, int M, int S, int d, int splits, int chunks) {
     const size_t rows = (size_t)units * M, Sr = (S + 3) / 4 * 4;
-    return chunks * ((size_t)units * S * 2 * d + rows * Sr * (group_splits(units, M, S, c_in, chunks) + 1) + 2 * ((rows + 3) / 4 * 4)) + (chunks + 2) * rows * 2 * d;
+    return chunks * ((size_t)units * S * 2 * d + rows * Sr * (splits + 1) + 2 * ((rows + 3) / 4 * 4)) + (chunks + 2) * rows * 2 * d;
 }
 
 }  // namespace
@@ -925,18 +925,23 @@ int simt_group_chunks(const lococo_handle* h, int L, int B, size_t* floats) {
     // M = 32, B = 142: 571 us a step at a time, 588 in one group). simt_group_supported draws a narrower line, by what the device runs at once.
     if ((int64_t)((c.M + B + 31) / 32 + (B + 31) / 32) * h->units > 6 * kSMs) return 0;
     // as many chunks as 128 MB hold
+    auto need = [&](int n) { return group_floats(h->units, c.M, c.M + B, c.head_dim, group_splits(h->units, c.M, c.M + B, c.c_in, n), n); };
     int n = std::min(chunks, 4096);
-    while (n > 1 && group_floats(h->units, c.M, c.M + B, c.head_dim, c.c_in, n) > (32u << 20)) n = std::min(n - 1, (n * 7 + 7) / 8);
+    while (n > 1 && need(n) > (32u << 20)) n = std::min(n - 1, (n * 7 + 7) / 8);
     if (n < 2) return 0;
-    *floats = group_floats(h->units, c.M, c.M + B, c.head_dim, c.c_in, n);
+    *floats = need(n);
     return n;
 }
 
-void simt_group_layout(BwdGroup& G, float* at) {
+size_t simt_group_layout(BwdGroup& G, float* scratch, size_t floats) {
     const BwdStep& p = G.first;
     const size_t rows = (size_t)p.units * p.M;
+    // The group that is left over at the front of a call may have fewer chunks than the others, and with fewer tiles its convolution is split
+    // further: only as far as the room goes. (As far as a whole group's always fits.)
     G.splits = group_splits(p.units, p.M, G.S, p.c_in, G.count);
-    auto take = [&](size_t floats) { float* r = at; at += floats; return r; };
+    while (G.splits > 1 && group_floats(p.units, p.M, G.S, p.d, G.splits, G.count) > floats) --G.splits;
+    float* at = scratch;
+    auto take = [&](size_t n) { float* r = at; at += n; return r; };
     G.attn = take((size_t)G.count * p.units * G.S * 2 * p.d);
     G.R = take(G.count * rows * G.Sr * G.splits);
     G.dA = take(G.count * rows * G.Sr);
@@ -944,6 +949,7 @@ void simt_group_layout(BwdGroup& G, float* at) {
     G.last = take(rows * 2 * p.d);
     G.s = take(G.count * ((rows + 3) / 4 * 4));
     G.inner = take(G.count * ((rows + 3) / 4 * 4));
+    return at - scratch;
 }
 
 int simt_backward_group(const BwdGroup& G, cudaStream_t st) {

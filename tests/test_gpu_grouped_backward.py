@@ -1,9 +1,11 @@
 """The fp32 backward pass of several chunks at a time (small problems): edges of its clusters, tiles and groups, against the
 float64 oracle's gradients."""
 import pytest
+import torch
 
 from paper_2406_05317_b200 import workloads as wl
-from tests.test_gpu_backward import check_backward
+from tests.helpers import to_device, to_host
+from tests.test_gpu_backward import check_backward, check_gradients
 
 pytestmark = pytest.mark.gpu
 
@@ -22,3 +24,50 @@ def test_grouped_backward(batch, heads, d, M, B, L, k, c_mult, per_head, bias):
     w = wl.Workload("grouped", 38, batch=batch, heads=heads, d=d, M=M, B=B, k=k, L=L, dtype="f32", weights_per_head=per_head, qkv_scale=1.0,
                     g_std=0.05, c_in_mult=c_mult)
     check_backward(w, bias=bias)
+
+
+class Training:
+    """A forward pass with its snapshots; backward passes of it with a scratch of the test's own."""
+
+    def __init__(self, w):
+        from paper_2406_05317_b200 import api
+        self.w, self.ctx = w, api.Lococo(w.batch, w.heads, w.d, w.M, w.k, w.B, dtype=torch.float32, c_in=w.c_in, weights_per_head=w.weights_per_head)
+        self.G, self.bias = wl.make_weights(w, with_bias=True)
+        self.ctx.set_weights(to_device(self.G, "f32"), to_device(self.bias, "f32"))
+        self.host = (*wl.make_qkv(w), *wl.make_loss_projections(w))
+        self.Q, self.K, self.V, self.PO, self.PK, self.PV = (to_device(x, "f32") for x in self.host)
+        self.O = torch.empty_like(self.Q)
+        caches = [torch.zeros(w.batch, w.heads, w.M, w.d, device="cuda") for _ in range(2)]
+        self.saved = torch.empty(self.ctx.saved_bytes(w.L, w.B), dtype=torch.uint8, device="cuda")
+        self.ctx.process_sequence(self.Q, self.K, self.V, w.B, self.O, *caches, 0, self.saved)
+        self.scratch_bytes = self.ctx.backward_scratch_bytes(w.L, w.B)
+
+    def backward(self, scratch):
+        """Gradients, and how many launches they took."""
+        grads = [torch.empty_like(self.Q) for _ in range(3)]
+        dG, dbias = torch.zeros(self.G.shape, device="cuda"), torch.zeros(self.bias.shape, device="cuda")
+        before = self.ctx.launch_count()
+        self.ctx.process_sequence_backward(self.Q, self.K, self.V, self.O, self.w.B, self.saved, self.PO, self.PK, self.PV, *grads, dG, dbias, scratch)
+        torch.cuda.synchronize()
+        return dict(zip(("dQ", "dK", "dV", "dG", "dbias"), map(to_host, (*grads, dG, dbias)))), self.ctx.launch_count() - before
+
+    def check(self, got, n, h):
+        """Unit (n, h) against the oracle: with a weight set per head and one sequence all of its gradients are its own."""
+        from oracle import lococo_oracle as orc
+        assert self.w.weights_per_head and self.w.batch == 1
+        Q, K, V, PO, PK, PV = (x[n, h] for x in self.host)
+        ref = orc.process_sequence_grad(Q, K, V, self.G[h], self.w.B, PO, PK, PV, bias=self.bias[h])
+        check_gradients(self.w, {"dQ": got["dQ"][n, h], "dK": got["dK"][n, h], "dV": got["dV"][n, h], "dG": got["dG"][h], "dbias": got["dbias"][h]},
+                        dict(zip(("dQ", "dK", "dV", "dG", "dbias"), ref)))
+
+
+def test_a_shorter_last_group_stays_inside_the_scratch():
+    # 111 chunks in groups of 28, 28, 28 and 27: the tiles of 27 are few enough for two partial sums of the convolution each, those of 28 are not.
+    w = wl.Workload("grouped_rest", 39, batch=1, heads=16, d=128, M=16, B=200, k=5, L=22200, dtype="f32", weights_per_head=True, qkv_scale=1.0, g_std=0.05)
+    t = Training(w)
+    room = torch.full((t.scratch_bytes + (16 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+    got, launches = t.backward(room[:t.scratch_bytes])
+    assert launches == 1 + 4 * 5
+    assert bool((room[t.scratch_bytes:] == 0x5A).all())
+    t.check(got, 0, 0)
+    t.check(got, 0, 15)

@@ -2,6 +2,8 @@
 (tests/cuda/fake_runtime.c). What a failed call leaves behind, by failing the n-th for every n; which launches may start early; and
 grids at the largest sizes."""
 import ctypes
+import os
+import random
 import subprocess
 
 import pytest
@@ -19,14 +21,18 @@ def fake(tmp_path_factory):
     src = build.PKG.parent / "tests" / "cuda" / "fake_runtime.c"
     obj = out.with_suffix(".o")
     subprocess.check_call(["gcc", "-O1", "-w", "-fPIC", "-c", str(src), "-o", str(obj)])
+    layout = out.with_name("group_layout.o")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "-I", str(build.INCLUDE),
+                           "-I", str(build.CSRC), "-c", str(src.with_name("group_layout.cpp")), "-o", str(layout)])
     # (its own names first: another CUDA runtime may be loaded in this process)
-    subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-o", str(out), str(obj), *map(str, objects)])
+    subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-o", str(out), str(obj), str(layout), *map(str, objects)])
     lib = ctypes.CDLL(str(out))
     lib.fake_stream.restype = ctypes.c_void_p
     lib.fake_calls.restype = ctypes.c_long
     lib.fake_fail_at.argtypes = [ctypes.c_long]
     lib.fake_joined.argtypes = [ctypes.c_void_p]
     lib.fake_capture.argtypes = [ctypes.c_ulonglong]
+    lib.fake_group_overrun.restype = ctypes.c_longlong
     from paper_2406_05317_b200 import api
     for name, args in api._SIGNATURES.items():
         getattr(lib, name).argtypes = args
@@ -134,3 +140,25 @@ def test_grids_of_many_weight_sets(fake, d, heads, k):
     assert fake.lococo_process_sequence_backward(handle, tokens, tokens, tokens, tokens, L, L, 0, at, tokens, cache, cache, tokens,
                                                  tokens, tokens, at, None, none, none, at, size.value, stream) == api.OK
     fake.lococo_destroy(handle)
+
+
+def test_every_group_of_a_backward_pass_fits_its_scratch(fake):
+    # A call's chunks go in groups of as many as 128 MB hold, and the group that is left over has fewer: fewer tiles, more
+    # partial sums of the convolution each.
+    from paper_2406_05317_b200 import api
+    rng = random.Random(4)
+    # sizes whose left-over group would be split further than a whole one: 27 chunks behind three groups of 28; and others
+    sizes = [(16, 128, 16, 128, 200, 22200), (1, 128, 16, 128, 5620, 39 * 5620), (4, 128, 16, 128, 1092, 68 * 1092), (12, 128, 16, 128, 196, 151 * 196),
+             (8, 128, 16, 128, 224, 391 * 224), (8, 64, 48, 64, 100, 12100)]
+    for _ in range(4000):
+        d = rng.choice([64, 128])
+        M = rng.randint(1, 6144 // d)
+        B = int(16 * 512 ** rng.random())
+        sizes.append((rng.choice([1, 2, 4, 8, 12, 16, 24, 32, 48]), d, M, d * rng.choice([1, 2]), B, B * rng.randint(2, 700) - rng.randint(0, B - 1)))
+    left_over = 0
+    for units, d, M, c_in, B, L in sizes:
+        cfg, chunks = api.Config(1, units, d, M, 5, c_in, 0, api.F32, 0.0, 1e-6, B, api.PATH_AUTO), ctypes.c_int()
+        over = fake.fake_group_overrun(ctypes.byref(cfg), L, B, ctypes.byref(chunks))
+        assert over in (0, -1), (units, d, M, c_in, B, L, over)
+        left_over += over == 0 and -(-L // B) % chunks.value != 0
+    assert left_over > 100
