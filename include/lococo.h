@@ -238,7 +238,10 @@ lococo_status lococo_process_sequence_host(lococo_handle* handle, const void* Q_
  * the gradient w.r.t. the cache the forward started from (rows at and beyond cache_len_in: zeros).
  * A sequence processed in several forward calls is differentiated call by call, last call first,
  * each call's dK_cache_in/dV_cache_in being the dK_cache_final/dV_cache_final of the call before it.
- * scratch: device memory of lococo_backward_scratch_bytes.
+ * scratch: device memory of lococo_backward_scratch_bytes, or less: that size holds up to 128 MB with which small fp32 problems
+ * take several chunks at a time. Without that room the same gradients are computed in smaller groups or a chunk at a time, and a scratch
+ * made for the longest sequence and the largest chunk serves all calls of the handle (LOCOCO_ERR_WORKSPACE: too small for a chunk
+ * at a time as well).
  */
 lococo_status lococo_backward_scratch_bytes(const lococo_handle* handle, int32_t L, int32_t B, size_t* out);
 lococo_status lococo_process_sequence_backward(lococo_handle* handle, lococo_tensor Q, lococo_tensor K,

@@ -107,12 +107,14 @@ View bdev(const lococo_tensor& t, int64_t tokens, size_t elt) {
 }
 
 struct Scratch {
-    size_t gK, gV, parts, dA, delta, tensor, group, total;
+    size_t gK, gV, parts, dA, delta, tensor, group;
+    size_t least, total;       // what some way of doing the call fits in; what the fastest takes
     size_t group_floats;       // room of the groups
     int group_chunks;          // chunks that one go of the CUDA cores can take (0: a step at a time)
 };
 
-Scratch scratch_layout(const lococo_handle* h, int L, int B) {
+// `bytes`: of the caller's scratch. With less than `total` groups are of fewer chunks, or there are none.
+Scratch scratch_layout(const lococo_handle* h, int L, int B, size_t bytes) {
     const lococo_config& c = h->cfg;
     const size_t units = h->units, Smax = (size_t)c.M + B;
     Scratch s{};
@@ -127,11 +129,13 @@ Scratch scratch_layout(const lococo_handle* h, int L, int B) {
         s.parts = take(simt_backward_parts_floats(h->units, c.M, B, c.head_dim) * sizeof(float));
         s.dA = take(units * c.M * ((Smax + 3) / 4 * 4) * sizeof(float));
         // (in the place of what single steps need: a call takes the one way or the other)
+        s.least = off;
         s.group = s.parts;
-        s.group_chunks = simt_group_chunks(h, L, B, &s.group_floats);
+        s.group_chunks = simt_group_chunks(h, L, B, bytes < s.group ? 0 : (bytes - s.group) / sizeof(float), &s.group_floats);
         off = std::max(off, s.group + align256(s.group_floats * sizeof(float)));
     }
     s.total = off;
+    if (s.least == 0) s.least = off;
     return s;
 }
 
@@ -141,7 +145,7 @@ extern "C" {
 
 lococo_status lococo_backward_scratch_bytes(const lococo_handle* h, int32_t L, int32_t B, size_t* out) {
     if (!h || !out || L < 1 || B < 1 || B > h->cfg.max_chunk) return LOCOCO_ERR_INVALID_ARG;
-    *out = scratch_layout(h, L, B).total;
+    *out = scratch_layout(h, L, B, SIZE_MAX).total;
     return LOCOCO_OK;
 }
 
@@ -166,8 +170,8 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
     if ((dKc_final.ptr && !bview_ok(dKc_final, e)) || (dVc_final.ptr && !bview_ok(dVc_final, e))) return LOCOCO_ERR_INVALID_ARG;
     if ((dKc_in.ptr && !bview_ok(dKc_in, e)) || (dVc_in.ptr && !bview_ok(dVc_in, e))) return LOCOCO_ERR_INVALID_ARG;
     if (dbias && !h->has_bias) return LOCOCO_ERR_INVALID_ARG;
-    const Scratch sl = scratch_layout(h, L, B);
-    if (scratch_bytes < sl.total) return LOCOCO_ERR_WORKSPACE;
+    const Scratch sl = scratch_layout(h, L, B, scratch_bytes);
+    if (scratch_bytes < sl.least) return LOCOCO_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char* sc = static_cast<char*>(scratch);
     float* gK = reinterpret_cast<float*>(sc + sl.gK);

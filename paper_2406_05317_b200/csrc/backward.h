@@ -56,11 +56,13 @@ struct BwdGroup {
     float* dA;                 // [count][units][M][Sr]
     float* last;               // [units][M][2 d]: the cache after the call's last chunk
 };
-// Chunks of a group (0: one step at a time is the way), and the floats of scratch that a group takes; both depend on the sizes alone.
-int simt_group_chunks(const lococo_handle* h, int L, int B, size_t* floats);
+// Chunks of a group (0: one step at a time is the way) where there is room for `room` floats, and the floats of scratch that a group takes; both
+// depend on the sizes alone.
+int simt_group_chunks(const lococo_handle* h, int L, int B, size_t room, size_t* floats);
 // Lays the arrays of G out in the `floats` at `scratch` (what simt_group_chunks said, or less chunks' worth of it), and says how many they take.
 size_t simt_group_layout(BwdGroup& G, float* scratch, size_t floats);
 bool simt_group_supported(const BwdGroup& G);      // (clusters of CTAs that this device can run, and not one after another)
+bool simt_group_possible(const lococo_handle* h, int B);      // ... that a device whose SMs form any clusters could run: where not, no scratch is set aside
 int simt_backward_group(const BwdGroup& G, cudaStream_t st);
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st);      // (simt_chain.cu: the part of a group that is a chain)
 

@@ -285,21 +285,26 @@ ClusterKernel chain_state[2];
 template <int D>
 int resident(int ctas) { return resident_clusters(chain_state[D == 128], chain_kernel<D>, kMaxSmem, ctas, kThreads); }
 
-// CTAs per unit (0: none fits) by the fewest estimated microseconds per step, and how many of these are not the step's work spread over all SMs
+// CTAs per unit (0: none fits) by the fewest estimated microseconds per step, and how many of these are not the step's work spread over all SMs.
+// clusters(ctas): how many clusters of that many CTAs run at once.
 struct ChainPlan { int ctas; double us, idle_us; };
-ChainPlan chain_plan(const BwdGroup& G) {
-    const BwdStep& p = G.first;
+template <typename Clusters>
+ChainPlan chain_plan(int units, int M, int d, int k, int c_in, const Clusters& clusters_of) {
     ChainPlan best{0, 1e30, 0};
-    for (int ctas = 1; ctas <= std::min(kMaxCluster, p.M); ctas = ctas < 8 ? 2 * ctas : ctas + 1) {
-        const ChainLayout lay = chain_layout(p.d, p.M, p.k, p.c_in, ctas);
-        if ((double)lay.slots * p.k * p.c_in * 4 > kMaxSmem || (size_t)lay.total * 4 > kMaxSmem) continue;
-        const int clusters = p.d == 128 ? resident<128>(ctas) : resident<64>(ctas);
+    for (int ctas = 1; ctas <= std::min(kMaxCluster, M); ctas = ctas < 8 ? 2 * ctas : ctas + 1) {
+        const ChainLayout lay = chain_layout(d, M, k, c_in, ctas);
+        if ((double)lay.slots * k * c_in * 4 > kMaxSmem || (size_t)lay.total * 4 > kMaxSmem) continue;
+        const int clusters = clusters_of(ctas);
         if (clusters == 0) continue;
-        const double per_slot = (double)p.M * (4.0 * p.d + (double)p.c_in * p.k) / 90e3;
-        const double us = (p.units + clusters - 1) / clusters * (2.0 + 0.03 * ctas + lay.slots * per_slot);
-        if (us < best.us) best = {ctas, us, us - per_slot * p.M * p.units / kSMs};
+        const double per_slot = (double)M * (4.0 * d + (double)c_in * k) / 90e3;
+        const double us = (units + clusters - 1) / clusters * (2.0 + 0.03 * ctas + lay.slots * per_slot);
+        if (us < best.us) best = {ctas, us, us - per_slot * M * units / kSMs};
     }
     return best;
+}
+ChainPlan chain_plan(const BwdGroup& G) {
+    const BwdStep& p = G.first;
+    return chain_plan(p.units, p.M, p.d, p.k, p.c_in, [&](int ctas) { return p.d == 128 ? resident<128>(ctas) : resident<64>(ctas); });
 }
 
 }  // namespace
@@ -308,11 +313,14 @@ ChainPlan chain_plan(const BwdGroup& G) {
 // for one another's rows, and the attention's blocks (per SM) no longer hide anything where they alone fill the chip. The weights are a
 // least-squares fit to 78 sizes (6 us per step off). d = 128, B = 100, a training step in groups / a step at a time, us: 32 units, M = 32, k = 5
 // 560 / 643; 96, M = 16 1029 / 1047; 24, M = 32, k = 11 612 / 667, 48 1083 / 984; 16, M = 48, k = 5 497 / 527, 32 830 / 781, 96 2178 / 1706.
-bool simt_group_supported(const BwdGroup& G) {
-    const BwdStep& p = G.first;
-    const ChainPlan plan = chain_plan(G);
-    const int attention_blocks = ((p.M + G.B + 31) / 32 + (G.B + 31) / 32) * p.units;
-    return plan.ctas > 0 && 1.9 * plan.idle_us + 4.6 * attention_blocks / kSMs * p.d / 128 <= 28.0;
+static bool group_pays(const ChainPlan& plan, int units, int M, int B, int d) {
+    const int attention_blocks = ((M + B + 31) / 32 + (B + 31) / 32) * units;
+    return plan.ctas > 0 && 1.9 * plan.idle_us + 4.6 * attention_blocks / kSMs * d / 128 <= 28.0;
+}
+bool simt_group_supported(const BwdGroup& G) { return group_pays(chain_plan(G), G.first.units, G.first.M, G.B, G.first.d); }
+bool simt_group_possible(const lococo_handle* h, int B) {
+    const lococo_config& c = h->cfg;
+    return group_pays(chain_plan(h->units, c.M, c.head_dim, c.k, c.c_in, [](int ctas) { return kSMs / ctas; }), h->units, c.M, B, c.head_dim);
 }
 
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st) {

@@ -9,13 +9,13 @@
 
 using namespace lococo;
 
-// Floats that the groups of a call of L tokens in chunks of B take beyond the room reserved for them: the most of any group
-// (0: all fit; -1: no groups at these sizes; -2: two arrays overlap). *chunks: of a whole group.
-extern "C" long long fake_group_overrun(const lococo_config* cfg, int L, int B, int* chunks) {
+// Floats that the groups of a call of L tokens in chunks of B, where there is room for `room` floats, take beyond what is reserved for them:
+// the most of any group (0: all fit; -1: no groups at these sizes; -2: two arrays overlap). *chunks: of a whole group.
+extern "C" long long fake_group_overrun(const lococo_config* cfg, int L, int B, size_t room, int* chunks) {
     lococo_handle* h = nullptr;
     if (lococo_create(cfg, &h) != LOCOCO_OK) return -3;
     size_t floats = 0;
-    const int most = simt_group_chunks(h, L, B, &floats), units = h->units;
+    const int most = simt_group_chunks(h, L, B, room, &floats), units = h->units;
     lococo_destroy(h);
     *chunks = most;
     if (most == 0) return -1;

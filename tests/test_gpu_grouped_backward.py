@@ -71,3 +71,20 @@ def test_a_shorter_last_group_stays_inside_the_scratch():
     assert bool((room[t.scratch_bytes:] == 0x5A).all())
     t.check(got, 0, 0)
     t.check(got, 0, 15)
+
+
+def test_less_scratch():
+    # Groups of as many chunks as the scratch holds; with what one chunk takes, and nothing more, a chunk at a time.
+    units, d, M, B, L = 8, 64, 48, 64, 777
+    t = Training(wl.Workload("grouped_less", 40, batch=1, heads=units, d=d, M=M, B=B, k=5, L=L, dtype="f32", weights_per_head=True, qkv_scale=1.0, g_std=0.05))
+    one = units * (M + B) * 2 * d                                   # a gradient of all rows of [cache; chunk]
+    least = sum((4 * n + 255) // 256 * 256 for n in (units * M * d, units * M * d, units * L, one * (1 + M // 16), units * M * (M + B)))
+    assert least < t.scratch_bytes
+    launches = []
+    for size in (t.scratch_bytes, t.scratch_bytes // 2, t.scratch_bytes // 4, least):
+        room = torch.full((size + (8 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+        got, n = t.backward(room[:size])
+        assert bool((room[size:] == 0x5A).all())
+        t.check(got, 0, 5)
+        launches.append(n)
+    assert launches[0] == 1 + 5 and launches[0] < launches[1] < launches[2] and launches[3] == 2 + 4 * 13

@@ -32,8 +32,9 @@ def fake(tmp_path_factory):
     lib.fake_fail_at.argtypes = [ctypes.c_long]
     lib.fake_joined.argtypes = [ctypes.c_void_p]
     lib.fake_capture.argtypes = [ctypes.c_ulonglong]
-    lib.fake_group_overrun.restype = ctypes.c_longlong
     from paper_2406_05317_b200 import api
+    lib.fake_group_overrun.restype = ctypes.c_longlong
+    lib.fake_group_overrun.argtypes = [ctypes.POINTER(api.Config), ctypes.c_int, ctypes.c_int, ctypes.c_size_t, ctypes.c_void_p]
     for name, args in api._SIGNATURES.items():
         getattr(lib, name).argtypes = args
     return lib
@@ -158,7 +159,41 @@ def test_every_group_of_a_backward_pass_fits_its_scratch(fake):
     left_over = 0
     for units, d, M, c_in, B, L in sizes:
         cfg, chunks = api.Config(1, units, d, M, 5, c_in, 0, api.F32, 0.0, 1e-6, B, api.PATH_AUTO), ctypes.c_int()
-        over = fake.fake_group_overrun(ctypes.byref(cfg), L, B, ctypes.byref(chunks))
-        assert over in (0, -1), (units, d, M, c_in, B, L, over)
-        left_over += over == 0 and -(-L // B) % chunks.value != 0
+        for room in (1 << 40, rng.randint(1, 1 << 25)):      # all that a call asks for; what a caller has
+            over = fake.fake_group_overrun(ctypes.byref(cfg), L, B, room, ctypes.byref(chunks))
+            assert over in (0, -1), (units, d, M, c_in, B, L, room, over)
+            left_over += over == 0 and -(-L // B) % chunks.value != 0
     assert left_over > 100
+
+
+def test_scratch_of_a_larger_call_serves_a_smaller_one(fake):
+    # A trainer's scratch is made once, for the longest sequence and the largest chunk.
+    from paper_2406_05317_b200 import api
+    rng, stream, at = random.Random(5), fake.fake_stream(), 1 << 30
+    none = api.Tensor(None, 0, 0, 0)
+    sizes = [(8, 64, 48, 12100, 100, 12200, 100), (8, 64, 48, 777, 64, 777, 512)]      # (L, B of the call; L, B that the scratch is made for)
+    for _ in range(300):
+        L, B = int(64 * 200 ** rng.random()), int(8 * 64 ** rng.random())
+        sizes.append((rng.choice([1, 4, 8, 16]), rng.choice([64, 128]), rng.randint(4, 100), L, B, int(L * rng.uniform(1, 3)), int(B * rng.uniform(1, 8))))
+    smaller = 0
+    for heads, d, M, L, B, L_most, B_most in sizes:
+        handle, size, whole = ctypes.c_void_p(), ctypes.c_size_t(), ctypes.c_size_t()
+        cfg = api.Config(1, heads, d, M, 5, d, 0, api.F32, 0.0, 1e-6, B_most, api.PATH_AUTO)
+        fake.fake_fail_at(0)
+        assert fake.lococo_create(ctypes.byref(cfg), ctypes.byref(handle)) == api.OK
+        assert fake.lococo_workspace_bytes(handle, ctypes.byref(size)) == api.OK
+        assert fake.lococo_set_workspace(handle, at, size.value, stream) == api.OK
+        assert fake.lococo_set_weights(handle, at, None, stream) == api.OK
+        assert fake.lococo_backward_scratch_bytes(handle, L, B, ctypes.byref(whole)) == api.OK
+        assert fake.lococo_backward_scratch_bytes(handle, L_most, B_most, ctypes.byref(size)) == api.OK
+        smaller += size.value < whole.value
+        tokens, cache = (api.Tensor(at, heads * n * d, n * d, d) for n in (L, M))
+
+        def backward(scratch):
+            return fake.lococo_process_sequence_backward(handle, tokens, tokens, tokens, tokens, L, B, 0, at, tokens, cache, cache, tokens, tokens, tokens,
+                                                         at, None, none, none, at, scratch, stream)
+
+        assert backward(size.value) == api.OK, (heads, d, M, L, B, L_most, B_most)
+        assert backward(4 * heads * (2 * M * d + L)) == api.ERR_WORKSPACE      # (no room for anything but the cache's gradients and delta)
+        fake.lococo_destroy(handle)
+    assert smaller > 5
