@@ -42,9 +42,9 @@ class Training:
         self.ctx.process_sequence(self.Q, self.K, self.V, w.B, self.O, *caches, 0, self.saved)
         self.scratch_bytes = self.ctx.backward_scratch_bytes(w.L, w.B)
 
-    def backward(self, scratch):
-        """Gradients, and how many launches they took."""
-        grads = [torch.empty_like(self.Q) for _ in range(3)]
+    def backward(self, scratch, in_place=False):
+        """Gradients, and how many launches they took. in_place: those of K and V take the place of K and V."""
+        grads = [torch.empty_like(self.Q), self.K, self.V] if in_place else [torch.empty_like(self.Q) for _ in range(3)]
         dG, dbias = torch.zeros(self.G.shape, device="cuda"), torch.zeros(self.bias.shape, device="cuda")
         before = self.ctx.launch_count()
         self.ctx.process_sequence_backward(self.Q, self.K, self.V, self.O, self.w.B, self.saved, self.PO, self.PK, self.PV, *grads, dG, dbias, scratch)
@@ -88,3 +88,16 @@ def test_less_scratch():
         t.check(got, 0, 5)
         launches.append(n)
     assert launches[0] == 1 + 5 and launches[0] < launches[1] < launches[2] and launches[3] == 2 + 4 * 13
+
+
+def test_gradients_in_the_place_of_keys_and_values():
+    # stacked input: dG reads both
+    w = wl.Workload("grouped_place", 41, batch=1, heads=4, d=64, M=32, B=50, k=7, L=333, dtype="f32", weights_per_head=True, qkv_scale=1.0, g_std=0.05,
+                    c_in_mult=2)
+    t = Training(w)
+    scratch = torch.empty(t.scratch_bytes, dtype=torch.uint8, device="cuda")
+    assert t.backward(scratch)[1] == 1 + 5
+    got, launches = t.backward(scratch, in_place=True)
+    assert launches == 2 + 4 * 7
+    for h in range(4):
+        t.check(got, 0, h)

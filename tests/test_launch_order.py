@@ -175,7 +175,7 @@ def test_scratch_of_a_larger_call_serves_a_smaller_one(fake):
     for _ in range(300):
         L, B = int(64 * 200 ** rng.random()), int(8 * 64 ** rng.random())
         sizes.append((rng.choice([1, 4, 8, 16]), rng.choice([64, 128]), rng.randint(4, 100), L, B, int(L * rng.uniform(1, 3)), int(B * rng.uniform(1, 8))))
-    smaller = 0
+    smaller = grouped = 0
     for heads, d, M, L, B, L_most, B_most in sizes:
         handle, size, whole = ctypes.c_void_p(), ctypes.c_size_t(), ctypes.c_size_t()
         cfg = api.Config(1, heads, d, M, 5, d, 0, api.F32, 0.0, 1e-6, B_most, api.PATH_AUTO)
@@ -188,12 +188,24 @@ def test_scratch_of_a_larger_call_serves_a_smaller_one(fake):
         assert fake.lococo_backward_scratch_bytes(handle, L_most, B_most, ctypes.byref(size)) == api.OK
         smaller += size.value < whole.value
         tokens, cache = (api.Tensor(at, heads * n * d, n * d, d) for n in (L, M))
+        grad = api.Tensor(2 * at, heads * L * d, L * d, d)
 
-        def backward(scratch):
-            return fake.lococo_process_sequence_backward(handle, tokens, tokens, tokens, tokens, L, B, 0, at, tokens, cache, cache, tokens, tokens, tokens,
-                                                         at, None, none, none, at, scratch, stream)
+        def backward(scratch, grads=(grad, grad, grad)):
+            before, after = ctypes.c_int64(), ctypes.c_int64()
+            fake.lococo_launch_count(handle, ctypes.byref(before))
+            status = fake.lococo_process_sequence_backward(handle, tokens, tokens, tokens, tokens, L, B, 0, at, tokens, cache, cache, *grads,
+                                                           at, None, none, none, at, scratch, stream)
+            fake.lococo_launch_count(handle, ctypes.byref(after))
+            launches.append(after.value - before.value)
+            return status
 
+        launches = []
         assert backward(size.value) == api.OK, (heads, d, M, L, B, L_most, B_most)
+        # gradients in the place of keys or values: a chunk at a time, which is done with a chunk's rows when it writes their gradients
+        assert backward(whole.value, (grad, tokens, grad)) == backward(whole.value, (grad, grad, tokens)) == api.OK
+        full = [min(M, n * B) + min(B, L - n * B) > M for n in range(-(-L // B))]
+        assert launches[1] == launches[2] == 2 + sum(4 if compress else 2 for compress in full)
+        grouped += launches[0] < launches[1]
         assert backward(4 * heads * (2 * M * d + L)) == api.ERR_WORKSPACE      # (no room for anything but the cache's gradients and delta)
         fake.lococo_destroy(handle)
-    assert smaller > 5
+    assert smaller > 5 and grouped > 50
