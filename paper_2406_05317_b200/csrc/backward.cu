@@ -216,7 +216,8 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
     // (A group's last launch writes dK and dV while it reads K and V for dG; single steps are done with a chunk's rows when they write
     // its gradients. A caller who wants them in place gets the latter.)
     auto in_place = [&](const lococo_tensor& t) { return t.ptr == K.ptr || t.ptr == V.ptr; };
-    const bool grouped = sl.group_chunks && !in_place(dK) && !in_place(dV) && simt_group_supported(G);
+    if (sl.group_chunks && !in_place(dK) && !in_place(dV)) G.ctas = simt_group_clusters(G);
+    const bool grouped = G.ctas > 0;
     // groups n0, n0 + group_chunks, ... from the last chunk back; the one that is left at the front may be shorter
     auto group_before = [&](int n) {
         G.count = std::min(n, sl.group_chunks);

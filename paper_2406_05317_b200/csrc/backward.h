@@ -43,6 +43,7 @@ struct BwdGroup {
     int64_t snap_step;         // floats between snapshots
     int S, Sr;                 // of a whole chunk on a full cache: the stride of positions in all arrays here
     int splits;                // partial sums of the recomputed convolution
+    int ctas;                  // CTAs per unit for the chain
     const void* g_packed;      // as in CompressParams
     const float* bias;
     float eps;
@@ -61,7 +62,7 @@ struct BwdGroup {
 int simt_group_chunks(const lococo_handle* h, int L, int B, size_t room, size_t* floats);
 // Lays the arrays of G out in the `floats` at `scratch` (what simt_group_chunks said, or less chunks' worth of it), and says how many they take.
 size_t simt_group_layout(BwdGroup& G, float* scratch, size_t floats);
-bool simt_group_supported(const BwdGroup& G);      // (clusters of CTAs that this device can run, and not one after another)
+int simt_group_clusters(const BwdGroup& G);        // CTAs per unit for the chain (0: clusters that this device would not run, or one after another)
 bool simt_group_possible(const lococo_handle* h, int B);      // ... that a device whose SMs form any clusters could run: where not, no scratch is set aside
 int simt_backward_group(const BwdGroup& G, cudaStream_t st);
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st);      // (simt_chain.cu: the part of a group that is a chain)

@@ -128,9 +128,12 @@ bool tensor_sequence_add(lococo_handle* h, const AttnParams& a, const CompressPa
 int tensor_sequence_launch(lococo_handle* h, cudaStream_t st, void* prof);
 void tensor_sequence_release(lococo_handle* h);
 
-// The whole chunk loop of a small fp32 problem in one launch (simt_loop.cu), and when that is the faster way.
-bool simt_loop_preferred(const lococo_handle* h, int L, int B);
-int simt_loop(lococo_handle* h, View q, View k, View v, int L, int B, View o, View kc, View vc, int c0, char* saved, size_t snap_step,
+// The whole chunk loop of a small fp32 problem in one launch (simt_loop.cu): how, where that is the faster way.
+struct LoopPlan {
+    int ctas, chain_warps, tile;      // CTAs per unit (0: not this way), warps that update the cache, convolution tile
+};
+LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B);
+int simt_loop(lococo_handle* h, const LoopPlan& plan, View q, View k, View v, int L, int B, View o, View kc, View vc, int c0, char* saved, size_t snap_step,
               size_t snap_all, cudaStream_t st);
 
 }  // namespace lococo

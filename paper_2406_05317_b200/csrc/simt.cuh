@@ -92,19 +92,24 @@ inline bool smem_limit(Kernel kernel, int bytes, bool (&done)[64]) {
 
 // A kernel launched as clusters of up to 16 CTAs: its per-device attributes, and how many clusters of each size a device runs at
 // the same time (a cluster lies within one group of SMs).
+constexpr int kMaxCluster = 16;
+inline int next_cluster(int ctas) { return ctas < 8 ? 2 * ctas : ctas + 1; }      // the sizes in use: 1, 2, 4, 8, 9 .. 16
 struct ClusterKernel {
-    bool smem[64] = {}, wide[64] = {};
-    std::atomic<int> resident[64][17] = {};
+    bool ready[64] = {};
+    std::atomic<bool> counted[64] = {};
+    std::atomic<int> resident[64][kMaxCluster + 1] = {};
 };
+// The current device, with the kernel's attributes set there; or -1
 template <typename Kernel>
-inline bool cluster_attributes(ClusterKernel& k, Kernel kernel, int max_smem) {
+inline int cluster_device(ClusterKernel& k, Kernel kernel, int max_smem) {
     int dev = -1;
-    if (!smem_limit(kernel, max_smem, k.smem) || cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (!k.wide[dev]) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
-        k.wide[dev] = true;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
+    if (!k.ready[dev]) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess ||
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return -1;
+        k.ready[dev] = true;
     }
-    return true;
+    return dev;
 }
 inline cudaLaunchAttribute cluster_of(int ctas) {
     cudaLaunchAttribute a;
@@ -113,16 +118,17 @@ inline cudaLaunchAttribute cluster_of(int ctas) {
     a.val.clusterDim.y = a.val.clusterDim.z = 1;
     return a;
 }
-// (0 where it cannot be told)
+// Clusters of every size (index: CTAs) that the current device runs at once (0: none, or it cannot be told), or nullptr. Asked of the runtime once per
+// device, for all sizes: plans are made in every call, and 24 such questions per call cost a one-chunk call 10 us of host time.
 template <typename Kernel>
-inline int resident_clusters(ClusterKernel& k, Kernel kernel, int max_smem, int ctas, int threads) {
-    int dev = -1;
-    if (!cluster_attributes(k, kernel, max_smem) || cudaGetDevice(&dev) != cudaSuccess) {
+inline const std::atomic<int>* resident_clusters(ClusterKernel& k, Kernel kernel, int max_smem, int threads) {
+    const int dev = cluster_device(k, kernel, max_smem);
+    if (dev < 0) {
         cudaGetLastError();
-        return 0;
+        return nullptr;
     }
-    int n = k.resident[dev][ctas].load(std::memory_order_relaxed);
-    if (n == 0) {
+    if (k.counted[dev].load(std::memory_order_acquire)) return k.resident[dev];
+    for (int ctas = 1; ctas <= kMaxCluster; ctas = next_cluster(ctas)) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(ctas);
         cfg.blockDim = dim3(threads);
@@ -130,17 +136,19 @@ inline int resident_clusters(ClusterKernel& k, Kernel kernel, int max_smem, int 
         cudaLaunchAttribute attr = cluster_of(ctas);
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
+        int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
             cudaGetLastError();
             n = 0;
         }
-        k.resident[dev][ctas].store(n, std::memory_order_relaxed);
+        k.resident[dev][ctas].store(n, std::memory_order_relaxed);      // (threads that come here together store the same)
     }
-    return n;
+    k.counted[dev].store(true, std::memory_order_release);
+    return k.resident[dev];
 }
 template <typename... Params, typename... Args>
 inline bool launch_clusters(ClusterKernel& k, void (*kernel)(Params...), int max_smem, int ctas, int clusters, int threads, size_t smem, cudaStream_t st, const Args&... args) {
-    if (!cluster_attributes(k, kernel, max_smem)) return false;
+    if (cluster_device(k, kernel, max_smem) < 0) return false;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(clusters * ctas);
     cfg.blockDim = dim3(threads);

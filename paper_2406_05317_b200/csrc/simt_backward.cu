@@ -923,7 +923,7 @@ int simt_group_chunks(const lococo_handle* h, int L, int B, size_t room, size_t*
     *floats = 0;
     if (c.dtype != LOCOCO_F32 || chunks < 2 || (size_t)c.M * c.head_dim > 6144 || !simt_group_possible(h, B)) return 0;      // (larger caches: not in simt_chain.cu's shared memory)
     // Where the attention's blocks of one chunk alone are more than six per SM, single steps are as fast and take less memory (96 units,
-    // M = 32, B = 142: 571 us a step at a time, 588 in one group). simt_group_supported draws a narrower line, by what the device runs at once.
+    // M = 32, B = 142: 571 us a step at a time, 588 in one group). simt_group_clusters draws a narrower line, by what the device runs at once.
     if ((int64_t)((c.M + B + 31) / 32 + (B + 31) / 32) * h->units > 6 * kSMs) return 0;
     // as many chunks as 128 MB hold, or the caller's scratch
     auto need = [&](int n) { return group_floats(h->units, c.M, c.M + B, c.head_dim, group_splits(h->units, c.M, c.M + B, c.c_in, n), n); };

@@ -24,7 +24,6 @@ using namespace simt;
 
 constexpr int kThreads = 512, kWarps = kThreads / 32;
 constexpr int kMaxSmem = 232448 - 128;
-constexpr int kMaxCluster = 16;
 constexpr int kShareWarps = 12;          // make a CTA's share of g'; the others fetch
 constexpr int kTA = 3, kTP = 4;          // slots x positions of a tile of dw: with the three <dw, w>, fifteen sums over the lanes
 
@@ -56,18 +55,12 @@ __host__ __device__ inline ChainLayout chain_layout(int d, int M, int k, int c_i
     return l;
 }
 
-struct ChainParams {
-    BwdGroup G;
-    int ctas;
-};
-
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1) chain_kernel(const __grid_constant__ ChainParams P) {
+__global__ void __launch_bounds__(kThreads, 1) chain_kernel(const __grid_constant__ BwdGroup G) {
     extern __shared__ __align__(16) float smem[];
     constexpr int kQ = D / 2, RS = 2 * D + 4;                     // quads of channels per row [keys | values]
-    const BwdGroup& G = P.G;
     const BwdStep& F = G.first;
-    const int ctas = P.ctas, rank = blockIdx.x % ctas, u = blockIdx.x / ctas, n = u / F.heads, h = u % F.heads;
+    const int ctas = G.ctas, rank = blockIdx.x % ctas, u = blockIdx.x / ctas, n = u / F.heads, h = u % F.heads;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int M = F.M, k = F.k, C = F.c_in, pad = (k - 1) / 2;
     const int i_begin = M * rank / ctas, slots = M * (rank + 1) / ctas - i_begin;
@@ -282,29 +275,23 @@ __global__ void __launch_bounds__(kThreads, 1) chain_kernel(const __grid_constan
 }
 
 ClusterKernel chain_state[2];
-template <int D>
-int resident(int ctas) { return resident_clusters(chain_state[D == 128], chain_kernel<D>, kMaxSmem, ctas, kThreads); }
 
 // CTAs per unit (0: none fits) by the fewest estimated microseconds per step, and how many of these are not the step's work spread over all SMs.
-// clusters(ctas): how many clusters of that many CTAs run at once.
+// resident[ctas]: how many clusters of that many CTAs run at once.
 struct ChainPlan { int ctas; double us, idle_us; };
-template <typename Clusters>
-ChainPlan chain_plan(int units, int M, int d, int k, int c_in, const Clusters& clusters_of) {
+template <typename Count>
+ChainPlan chain_plan(int units, int M, int d, int k, int c_in, const Count* resident) {
     ChainPlan best{0, 1e30, 0};
-    for (int ctas = 1; ctas <= std::min(kMaxCluster, M); ctas = ctas < 8 ? 2 * ctas : ctas + 1) {
+    for (int ctas = 1; resident && ctas <= std::min(kMaxCluster, M); ctas = next_cluster(ctas)) {
         const ChainLayout lay = chain_layout(d, M, k, c_in, ctas);
         if ((double)lay.slots * k * c_in * 4 > kMaxSmem || (size_t)lay.total * 4 > kMaxSmem) continue;
-        const int clusters = clusters_of(ctas);
+        const int clusters = resident[ctas];
         if (clusters == 0) continue;
         const double per_slot = (double)M * (4.0 * d + (double)c_in * k) / 90e3;
         const double us = (units + clusters - 1) / clusters * (2.0 + 0.03 * ctas + lay.slots * per_slot);
         if (us < best.us) best = {ctas, us, us - per_slot * M * units / kSMs};
     }
     return best;
-}
-ChainPlan chain_plan(const BwdGroup& G) {
-    const BwdStep& p = G.first;
-    return chain_plan(p.units, p.M, p.d, p.k, p.c_in, [&](int ctas) { return p.d == 128 ? resident<128>(ctas) : resident<64>(ctas); });
 }
 
 }  // namespace
@@ -317,19 +304,25 @@ static bool group_pays(const ChainPlan& plan, int units, int M, int B, int d) {
     const int attention_blocks = ((M + B + 31) / 32 + (B + 31) / 32) * units;
     return plan.ctas > 0 && 1.9 * plan.idle_us + 4.6 * attention_blocks / kSMs * d / 128 <= 28.0;
 }
-bool simt_group_supported(const BwdGroup& G) { return group_pays(chain_plan(G), G.first.units, G.first.M, G.B, G.first.d); }
+int simt_group_clusters(const BwdGroup& G) {
+    const BwdStep& p = G.first;
+    const std::atomic<int>* resident = p.d == 128 ? resident_clusters(chain_state[1], chain_kernel<128>, kMaxSmem, kThreads)
+                                     : resident_clusters(chain_state[0], chain_kernel<64>, kMaxSmem, kThreads);
+    const ChainPlan plan = chain_plan(p.units, p.M, p.d, p.k, p.c_in, resident);
+    return group_pays(plan, p.units, p.M, G.B, p.d) ? plan.ctas : 0;
+}
 bool simt_group_possible(const lococo_handle* h, int B) {
     const lococo_config& c = h->cfg;
-    return group_pays(chain_plan(h->units, c.M, c.head_dim, c.k, c.c_in, [](int ctas) { return kSMs / ctas; }), h->units, c.M, B, c.head_dim);
+    int most[kMaxCluster + 1];
+    for (int ctas = 1; ctas <= kMaxCluster; ++ctas) most[ctas] = kSMs / ctas;
+    return group_pays(chain_plan(h->units, c.M, c.head_dim, c.k, c.c_in, most), h->units, c.M, B, c.head_dim);
 }
 
 int simt_backward_chain(const BwdGroup& G, cudaStream_t st) {
-    ChainParams P{G, chain_plan(G).ctas};
-    if (P.ctas == 0) return -1;
     const BwdStep& p = G.first;
-    const size_t smem = (size_t)chain_layout(p.d, p.M, p.k, p.c_in, P.ctas).total * 4;
-    return (p.d == 128 ? launch_clusters(chain_state[1], chain_kernel<128>, kMaxSmem, P.ctas, p.units, kThreads, smem, st, P)
-                       : launch_clusters(chain_state[0], chain_kernel<64>, kMaxSmem, P.ctas, p.units, kThreads, smem, st, P)) ? 1 : -1;
+    const size_t smem = (size_t)chain_layout(p.d, p.M, p.k, p.c_in, G.ctas).total * 4;
+    return (p.d == 128 ? launch_clusters(chain_state[1], chain_kernel<128>, kMaxSmem, G.ctas, p.units, kThreads, smem, st, G)
+                       : launch_clusters(chain_state[0], chain_kernel<64>, kMaxSmem, G.ctas, p.units, kThreads, smem, st, G)) ? 1 : -1;
 }
 
 }  // namespace lococo

@@ -30,7 +30,6 @@ using namespace simt;
 
 constexpr int kThreads = 512, kWarps = kThreads / 32;
 constexpr int kMaxSmem = 232448 - 128;   // dynamic shared memory: 227 KB less the kernel's few static words
-constexpr int kMaxCluster = 16;
 
 struct LoopParams {
     View q, k, v, o, k_cache, v_cache;
@@ -421,16 +420,14 @@ int launch_loop(const LoopParams& P, int units, size_t smem, cudaStream_t st) {
 
 ClusterKernel loop_state;      // of the kernel that is asked how many clusters fit (all forms need an SM per CTA)
 
-struct LoopPlan {
-    int ctas, chain_warps, tile;     // (ctas 0: not this way)
-};
+}  // namespace
 
 // The plan, and the rule: fp32, [cache; chunk] in one SM's shared memory, and a chunk estimated faster than as launches over the whole
 // chip. Both estimates (us per chunk) are fitted to 44 shapes on a B200, every cluster size each, half of them within 10 % of the one
 // for clusters; the launches are slowest where a tile's channels and taps are many. Measured, launches / this, us per call: 256 tokens of
 // one unit, M = B = 16, d = 64, k = 5 263 / 41; of 148 units 383 / 69; 777 tokens of 8 units, M = 48, B = 100 180 / 72; 85 tokens of one unit,
 // M = B = 16, d = 128, k = 25 248 / 31; 349 tokens of 16 units, M = B = 64, k = 25 513 / 170. In no shape that fits were the launches faster.
-LoopPlan loop_plan(const lococo_handle* h, int L, int B) {
+LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B) {
     const lococo_config& c = h->cfg;
     LoopPlan best{0, 0, 0};
     if (c.dtype != LOCOCO_F32) return best;
@@ -438,8 +435,9 @@ LoopPlan loop_plan(const lococo_handle* h, int L, int B) {
     const double S = (double)c.M + B, keys = c.M + 0.5 * B, d2 = 2.0 * c.head_dim, taps = (double)c.c_in * c.k;
     if (2.0 * S * d2 * 4 > kMaxSmem) return best;
     double least = 11.0 + 0.012 * taps + h->units * (c.M * S * (taps + d2) + B * keys * d2) / (kSMs * 150000.0);
-    for (int ctas = 1; ctas <= std::min(kMaxCluster, c.M); ctas = ctas < 8 ? 2 * ctas : ctas + 1) {
-        const int slots = (c.M + ctas - 1) / ctas, queries = (B + ctas - 1) / ctas, clusters = resident_clusters(loop_state, small_loop_kernel<64, 16>, kMaxSmem, ctas, kThreads);
+    const std::atomic<int>* resident = resident_clusters(loop_state, small_loop_kernel<64, 16>, kMaxSmem, kThreads);
+    for (int ctas = 1; resident && ctas <= std::min(kMaxCluster, c.M); ctas = next_cluster(ctas)) {
+        const int slots = (c.M + ctas - 1) / ctas, queries = (B + ctas - 1) / ctas, clusters = resident[ctas];
         const double conv = slots * S * taps, blends = slots * S * d2, attention = queries * keys * d2;
         LoopPlan p{ctas, std::min(12, std::max(4, 2 * (int)(0.5 * kWarps * (conv + blends) / (conv + blends + 1.3 * attention) + 0.5))), 3};
         const LoopLayout lay = loop_layout(c.head_dim, c.M, B, c.k, c.c_in, ctas, kWarps - p.chain_warps);
@@ -461,11 +459,7 @@ LoopPlan loop_plan(const lococo_handle* h, int L, int B) {
     return best;
 }
 
-}  // namespace
-
-bool simt_loop_preferred(const lococo_handle* h, int L, int B) { return loop_plan(h, L, B).ctas > 0; }
-
-int simt_loop(lococo_handle* h, View q, View k, View v, int L, int B, View o, View kc, View vc, int c0, char* saved, size_t snap_step,
+int simt_loop(lococo_handle* h, const LoopPlan& plan, View q, View k, View v, int L, int B, View o, View kc, View vc, int c0, char* saved, size_t snap_step,
               size_t snap_all, cudaStream_t st) {
     const lococo_config& c = h->cfg;
     LoopParams P{};
@@ -476,7 +470,6 @@ int simt_loop(lococo_handle* h, View q, View k, View v, int L, int B, View o, Vi
     P.bias = h->has_bias ? reinterpret_cast<const float*>(h->ws + h->off_bias) : nullptr;
     P.eps = c.norm_eps;
     P.scale = h->scale;
-    const LoopPlan plan = loop_plan(h, L, B);
     P.ctas = plan.ctas; P.chain_warps = plan.chain_warps; P.tile = plan.tile;
     if (saved) {
         P.snap_k = reinterpret_cast<float*>(saved);

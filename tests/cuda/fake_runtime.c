@@ -89,12 +89,14 @@ void __cudaRegisterVar(void) {}
 
 static int encode(void) { return 0; }
 int cudaGetDriverEntryPoint(const char* name, void** f, unsigned long long flags, int* found) { (void)name; (void)flags; *f = (void*)encode; *found = 0; return 0; }
-int cudaGetDevice(int* d) { *d = 0; return 0; }
+static long queries;               /* questions about the device */
+long fake_queries(void) { long n = queries; queries = 0; return n; }
+int cudaGetDevice(int* d) { ++queries; *d = 0; return 0; }
 int cudaDeviceGetAttribute(int* v, int a, int d) { (void)a; (void)d; *v = 148; return 0; }
-int cudaFuncSetAttribute(const void* f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
+int cudaFuncSetAttribute(const void* f, int a, int v) { ++queries; (void)f; (void)a; (void)v; return 0; }
 int cudaGetLastError(void) { int r = last_error; last_error = 0; return r; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int t, size_t m, unsigned fl) { (void)f; (void)t; (void)m; (void)fl; *n = 1; return 0; }
-int cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* c) { (void)f; (void)c; *n = 33; return 0; }
+int cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* c) { ++queries; (void)f; (void)c; *n = 33; return 0; }
 int cudaStreamIsCapturing(void* s, int* v) { (void)s; *v = capture != 0; return 0; }
 int cudaStreamGetCaptureInfo_v2(void* s, int* v, unsigned long long* id, void* g, void* d, void* n) {
     (void)s; (void)g; (void)d; (void)n;

@@ -28,7 +28,7 @@ def fake(tmp_path_factory):
     subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-o", str(out), str(obj), str(layout), *map(str, objects)])
     lib = ctypes.CDLL(str(out))
     lib.fake_stream.restype = ctypes.c_void_p
-    lib.fake_calls.restype = ctypes.c_long
+    lib.fake_calls.restype = lib.fake_queries.restype = ctypes.c_long
     lib.fake_fail_at.argtypes = [ctypes.c_long]
     lib.fake_joined.argtypes = [ctypes.c_void_p]
     lib.fake_capture.argtypes = [ctypes.c_ulonglong]
@@ -209,3 +209,23 @@ def test_scratch_of_a_larger_call_serves_a_smaller_one(fake):
         assert backward(4 * heads * (2 * M * d + L)) == api.ERR_WORKSPACE      # (no room for anything but the cache's gradients and delta)
         fake.lococo_destroy(handle)
     assert smaller > 5 and grouped > 50
+
+
+def test_a_small_call_asks_the_device_little(fake):
+    # A one-chunk call is a launch of a few microseconds: what its plan needs to know of the device is asked in the first call.
+    from paper_2406_05317_b200 import api
+    stream, at, handle, size = fake.fake_stream(), 1 << 30, ctypes.c_void_p(), ctypes.c_size_t()
+    cfg = api.Config(1, 4, 64, 32, 5, 64, 0, api.F32, 0.0, 1e-6, 16, api.PATH_AUTO)
+    fake.fake_fail_at(0)
+    assert fake.lococo_create(ctypes.byref(cfg), ctypes.byref(handle)) == api.OK
+    assert fake.lococo_workspace_bytes(handle, ctypes.byref(size)) == api.OK
+    assert fake.lococo_set_workspace(handle, at, size.value, stream) == api.OK
+    assert fake.lococo_set_weights(handle, at, None, stream) == api.OK
+    view = lambda ptr, n: api.Tensor(ptr, 4 * n * 64, n * 64, 64)
+    for i in range(3):                 # (outputs of its own each time: nothing is replayed)
+        c, x = ctypes.c_int32(32), view(at, 16)
+        fake.fake_queries()
+        assert fake.lococo_process_sequence(handle, x, x, x, 16, 16, view(at * (2 + i), 16), view(at * 8, 32), view(at * 9, 32), ctypes.byref(c), None, stream) == api.OK
+        asked = fake.fake_queries()
+        assert i == 0 or asked <= 2, asked
+    fake.lococo_destroy(handle)
