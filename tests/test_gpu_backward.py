@@ -244,3 +244,13 @@ def test_backward_of_views_shared_by_heads_and_reversed(d, M, B, dtype):
     assert all(torch.equal(a, b) for a, b in zip(want, run(shared_Q, shared_dO, shared_Q, shared_dO)))
     turn = lambda t: Flipped(t.flip(0, 1).contiguous())
     assert all(torch.equal(a, b) for a, b in zip(want, run(own_Q, own_dO, turn(own_Q), turn(own_dO))))
+
+
+@pytest.mark.parametrize("d,M,B", [
+    (128, 128, 64), (128, 128, 130), (128, 128, 450),     # one, three and eight tiles of queries: P in the place of scores that two tiles on take again
+    (128, 40, 330),                                       # two terms
+    (64, 128, 700),
+])
+def test_keys_side_over_query_tiles(d, M, B):
+    w = wl.Workload("bwd_tiles", 42, batch=1, heads=2, d=d, M=M, B=B, k=5, L=2 * B + 50, dtype="bf16", weights_per_head=False, qkv_scale=0.3, g_std=0.02)
+    check_backward(w)
