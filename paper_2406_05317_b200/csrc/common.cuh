@@ -107,6 +107,7 @@ struct AttnParams {
 struct FillParams {
     View src_k, src_v, dst_k, dst_v;  // src rows 0..b-1 -> dst rows c..c+b-1
     int heads, units, d, c, b;
+    int late = 0;          // 1: the next launch is let in when the blocks end, not when they start
 };
 
 // CUDA-core kernels (simt_forward.cu). Each returns the number of kernels launched, or -1.

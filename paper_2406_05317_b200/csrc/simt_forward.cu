@@ -54,7 +54,8 @@ __global__ void to_f32_kernel(const T* __restrict__ in, float* __restrict__ out,
 // ------------------------------------------------------------------ fill branch
 template <typename T>
 __global__ void fill_kernel(FillParams p) {
-    start_and_wait();
+    if (!p.late) start_next();
+    wait_for_previous();
     const int u = blockIdx.y, n = u / p.heads, h = u % p.heads;
     const int vec = 16 / sizeof(T), per_row = p.d / vec;
     const int total = p.b * per_row;
