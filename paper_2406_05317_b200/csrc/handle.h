@@ -132,7 +132,7 @@ void tensor_sequence_release(lococo_handle* h);
 struct LoopPlan {
     int ctas, chain_warps, tile;      // CTAs per unit (0: not this way), warps that update the cache, convolution tile
 };
-LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B);
+LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B, int c0);
 int simt_loop(lococo_handle* h, const LoopPlan& plan, View q, View k, View v, int L, int B, View o, View kc, View vc, int c0, char* saved, size_t snap_step,
               size_t snap_all, cudaStream_t st);
 

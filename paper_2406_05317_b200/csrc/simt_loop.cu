@@ -17,6 +17,7 @@
 // of 4 47, of 2 56, one 66; 148 units, one each 81 -> 69); 777 tokens of 8 units, M = 48, B = 100 180 (launches) -> 72 (10 CTAs).
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -422,19 +423,32 @@ ClusterKernel loop_state;      // of the kernel that is asked how many clusters 
 
 }  // namespace
 
-// The plan, and the rule: fp32, [cache; chunk] in one SM's shared memory, and a chunk estimated faster than as launches over the whole
-// chip. Both estimates (us per chunk) are fitted to 44 shapes on a B200, every cluster size each, half of them within 10 % of the one
-// for clusters; the launches are slowest where a tile's channels and taps are many. Measured, launches / this, us per call: 256 tokens of
-// one unit, M = B = 16, d = 64, k = 5 263 / 41; of 148 units 383 / 69; 777 tokens of 8 units, M = 48, B = 100 180 / 72; 85 tokens of one unit,
-// M = B = 16, d = 128, k = 25 248 / 31; 349 tokens of 16 units, M = B = 64, k = 25 513 / 170. In no shape that fits were the launches faster.
-LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B) {
+// The plan, and the rule: fp32, [cache; chunk] in one SM's shared memory, and a call estimated faster than as launches over the whole chip. A fill
+// step is a short launch or two there, but here every cluster of a unit takes its turn; a compress step is mostly work that launches do in tiles
+// of 4096 logits and blocks of 32 queries, however few are needed. Both estimates are in us:
+//   here      3 + rounds of clusters x (2.6 for zeros and weights, 2.4 and the work's share per compress step, 1.5 and the attention per fill step)
+//   launches  1.4 + per step the attention's rounds of one block per SM; per fill step 3.6, per compress step the convolution's and the blends' rounds
+// A compress step here is fitted to 44 shapes with every cluster size each, the rest to 260 calls both ways (units 1 to 2000, M and B up to 110
+// and 150, one to twelve chunks, from empty and full caches). Launches / this, us per call: 256 tokens of one unit, M = B = 16, d = 64, k = 5
+// 263 / 41; 777 tokens of 8 units, M = 48, B = 100 180 / 72; two chunks of 16 of 1600 units, M = 8, d = 128, k = 5 697 / 122; and by launches:
+// 8 tokens that fill a cache of 48, 32 units, d = 128 10.4 / 18.6; one of 310, M = 24 18.6 / 105.
+LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B, int c0) {
     const lococo_config& c = h->cfg;
     LoopPlan best{0, 0, 0};
     if (c.dtype != LOCOCO_F32) return best;
     B = std::min(B, L);
     const double S = (double)c.M + B, keys = c.M + 0.5 * B, d2 = 2.0 * c.head_dim, taps = (double)c.c_in * c.k;
     if (2.0 * S * d2 * 4 > kMaxSmem) return best;
-    double least = 11.0 + 0.012 * taps + h->units * (c.M * S * (taps + d2) + B * keys * d2) / (kSMs * 150000.0);
+    const int chunks = (L + B - 1) / B, fills = c0 + L <= c.M ? chunks : std::min(chunks, (c.M - c0) / B), compresses = chunks - fills;
+    const double fill_keys = c0 + 0.5 * B * fills;
+    double least;
+    {
+        const int OT = slot_tile(c.M), PT = 4096 / OT;
+        const double tiles = (double)(((int)S + PT - 1) / PT) * ((c.M + OT - 1) / OT) * h->units, splits = std::max(1.0, std::min(std::floor(6 * kSMs / tiles), c.c_in / 32.0));
+        const double conv = taps * std::max(1 / splits, tiles / (4 * kSMs)), blends = std::floor((S + 63) / 64) * std::max(1.0, (c.M + 15) / 16 * d2 / 64 * h->units / (6 * kSMs));
+        auto attention = [&](double n) { return 3.2 * std::max(1.0, (double)h->units * ((B + 31) / 32) / kSMs) * (1 + std::floor(n / 64)) * c.head_dim / 64; };
+        least = 1.4 + fills * (3.6 + attention(fill_keys)) + compresses * (0.094 * conv + 5.6 * blends + attention(S));
+    }
     const std::atomic<int>* resident = resident_clusters(loop_state, small_loop_kernel<64, 16>, kMaxSmem, kThreads);
     for (int ctas = 1; resident && ctas <= std::min(kMaxCluster, c.M); ctas = next_cluster(ctas)) {
         const int slots = (c.M + ctas - 1) / ctas, queries = (B + ctas - 1) / ctas, clusters = resident[ctas];
@@ -442,7 +456,8 @@ LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B) {
         LoopPlan p{ctas, std::min(12, std::max(4, 2 * (int)(0.5 * kWarps * (conv + blends) / (conv + blends + 1.3 * attention) + 0.5))), 3};
         const LoopLayout lay = loop_layout(c.head_dim, c.M, B, c.k, c.c_in, ctas, kWarps - p.chain_warps);
         if (clusters == 0 || (double)slots * taps * 4 > kMaxSmem || (size_t)lay.total * 4 > kMaxSmem) continue;
-        const double t = (h->units + clusters - 1) / clusters * (2.4 + 0.025 * ctas + conv / 109e3 + blends / 240e3 + attention / 91e3);
+        const double compress = 2.4 + 0.025 * ctas + conv / 109e3 + blends / 240e3 + attention / 91e3, fill = 1.5 + queries * fill_keys * d2 / 9500;
+        const double t = 3 + (h->units + clusters - 1) / clusters * (2.6 + compresses * compress + fills * fill);
         if (t >= least) continue;
         least = t;
         // Tiles of 2 x 4 while that is one round of the chain's lanes; else 8 positions wide, of as many slots as waste least

@@ -96,7 +96,13 @@ int cudaDeviceGetAttribute(int* v, int a, int d) { (void)a; (void)d; *v = 148; r
 int cudaFuncSetAttribute(const void* f, int a, int v) { ++queries; (void)f; (void)a; (void)v; return 0; }
 int cudaGetLastError(void) { int r = last_error; last_error = 0; return r; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int t, size_t m, unsigned fl) { (void)f; (void)t; (void)m; (void)fl; *n = 1; return 0; }
-int cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* c) { ++queries; (void)f; (void)c; *n = 33; return 0; }
+int cudaOccupancyMaxActiveClusters(int* n, const void* f, const LaunchConfig* c) {      /* as a B200 with one CTA per SM */
+    static const int most[17] = {0, 148, 74, 0, 33, 0, 0, 0, 15, 15, 11, 7, 7, 7, 7, 7, 7};
+    (void)f;
+    ++queries;
+    *n = most[*(const unsigned*)c->attrs[0].value];      /* (the cluster's extent is the only attribute) */
+    return 0;
+}
 int cudaStreamIsCapturing(void* s, int* v) { (void)s; *v = capture != 0; return 0; }
 int cudaStreamGetCaptureInfo_v2(void* s, int* v, unsigned long long* id, void* g, void* d, void* n) {
     (void)s; (void)g; (void)d; (void)n;

@@ -229,3 +229,32 @@ def test_a_small_call_asks_the_device_little(fake):
         asked = fake.fake_queries()
         assert i == 0 or asked <= 2, asked
     fake.lococo_destroy(handle)
+
+
+@pytest.mark.parametrize("units,d,M,B,L,k,c_mult,cache_len,one_launch", [
+    (1, 64, 16, 16, 256, 5, 1, 0, True),
+    (1600, 128, 8, 16, 32, 5, 1, 8, True),        # many units of few slots: blocks and tiles that the launches fill to a tenth
+    (1600, 64, 4, 4, 12, 5, 1, 0, True),
+    (1600, 64, 24, 4, 4, 1, 1, 24, True),
+    (32, 128, 48, 8, 8, 9, 2, 0, False),          # chunks that only fill the cache, with weights that nobody needs
+    (310, 128, 24, 1, 1, 31, 1, 0, False),
+    (1310, 128, 87, 3, 18, 3, 1, 0, False),
+    (1932, 128, 29, 2, 4, 9, 2, 29, True),
+])
+def test_way_of_a_small_fp32_loop(fake, units, d, M, B, L, k, c_mult, cache_len, one_launch):
+    from paper_2406_05317_b200 import api
+    stream, at, handle, size = fake.fake_stream(), 1 << 30, ctypes.c_void_p(), ctypes.c_size_t()
+    cfg = api.Config(1, units, d, M, k, c_mult * d, 0, api.F32, 0.0, 1e-6, B, api.PATH_AUTO)
+    fake.fake_fail_at(0)
+    assert fake.lococo_create(ctypes.byref(cfg), ctypes.byref(handle)) == api.OK
+    assert fake.lococo_workspace_bytes(handle, ctypes.byref(size)) == api.OK
+    assert fake.lococo_set_workspace(handle, at, size.value, stream) == api.OK
+    assert fake.lococo_set_weights(handle, at, None, stream) == api.OK
+    view = lambda ptr, n: api.Tensor(ptr, units * n * d, n * d, d)
+    c, before, after = ctypes.c_int32(cache_len), ctypes.c_int64(), ctypes.c_int64()
+    fake.lococo_launch_count(handle, ctypes.byref(before))
+    assert fake.lococo_process_sequence(handle, *[view(at, L)] * 3, L, B, view(2 * at, L), view(8 * at, M), view(9 * at, M), ctypes.byref(c), None, stream) == api.OK
+    assert c.value == min(M, cache_len + L)
+    fake.lococo_launch_count(handle, ctypes.byref(after))
+    assert (after.value - before.value == 1) == one_launch
+    fake.lococo_destroy(handle)
