@@ -216,7 +216,11 @@ lococo_status lococo_process_sequence_backward(lococo_handle* h, lococo_tensor Q
     // (A group's last launch writes dK and dV while it reads K and V for dG; single steps are done with a chunk's rows when they write
     // its gradients. A caller who wants them in place gets the latter.)
     auto in_place = [&](const lococo_tensor& t) { return t.ptr == K.ptr || t.ptr == V.ptr; };
-    if (sl.group_chunks && !in_place(dK) && !in_place(dV)) G.ctas = simt_group_clusters(G);
+    // (Groups take the chain through the cache apart, and with fewer than two compress steps there is none. us, in a group / a step at a time: one
+    // fill step and one compress step, 127 units, d = 128, M = 14, B = 8 221 / 172, 4 units, M = 6, B = 4 60 / 50; three fill steps before it, 144
+    // units, d = 64 108 / 82; two compress steps, 3 units, d = 64, M = 8, B = 51 81 / 118, 42 units, d = 128, M = 20, B = 121 218 / 209.)
+    const int fills = cache_len_in + L <= cfg.M ? n_chunks : (cfg.M - cache_len_in) / B;
+    if (sl.group_chunks && n_chunks - fills >= 2 && !in_place(dK) && !in_place(dV)) G.ctas = simt_group_clusters(G);
     const bool grouped = G.ctas > 0;
     // groups n0, n0 + group_chunks, ... from the last chunk back; the one that is left at the front may be shorter
     auto group_before = [&](int n) {

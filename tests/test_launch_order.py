@@ -205,6 +205,8 @@ def test_scratch_of_a_larger_call_serves_a_smaller_one(fake):
         assert backward(whole.value, (grad, tokens, grad)) == backward(whole.value, (grad, grad, tokens)) == api.OK
         full = [min(M, n * B) + min(B, L - n * B) > M for n in range(-(-L // B))]
         assert launches[1] == launches[2] == 2 + sum(4 if compress else 2 for compress in full)
+        # nor is there a chain to take apart with fewer than two compress steps
+        assert launches[0] == launches[1] or sum(full) >= 2
         grouped += launches[0] < launches[1]
         assert backward(4 * heads * (2 * M * d + L)) == api.ERR_WORKSPACE      # (no room for anything but the cache's gradients and delta)
         fake.lococo_destroy(handle)
