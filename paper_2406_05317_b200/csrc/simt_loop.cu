@@ -429,9 +429,10 @@ ClusterKernel loop_state;      // of the kernel that is asked how many clusters 
 //   here      3 + rounds of clusters x (2.6 for zeros and weights, 2.4 and the work's share per compress step, 1.5 and the attention per fill step)
 //   launches  1.4 + per step the attention's rounds of one block per SM; per fill step 3.6, per compress step the convolution's and the blends' rounds
 // A compress step here is fitted to 44 shapes with every cluster size each, the rest to 260 calls both ways (units 1 to 2000, M and B up to 110
-// and 150, one to twelve chunks, from empty and full caches). Launches / this, us per call: 256 tokens of one unit, M = B = 16, d = 64, k = 5
-// 263 / 41; 777 tokens of 8 units, M = 48, B = 100 180 / 72; two chunks of 16 of 1600 units, M = 8, d = 128, k = 5 697 / 122; and by launches:
-// 8 tokens that fill a cache of 48, 32 units, d = 128 10.4 / 18.6; one of 310, M = 24 18.6 / 105.
+// and 150, one to twelve chunks, from empty and full caches); of 220 others, 212 go the way that is within 2 % of the faster one, the worst takes
+// twice as long (617 units, M = 54, twelve chunks of 2: 3715 by launches, 1759 here). Launches / this, us per call: 256 tokens of one unit, M = B = 16, d = 64, k = 5
+// 263 / 41; 777 tokens of 8 units, M = 48, B = 100 180 / 72; two chunks of 16 of 1600 units, M = 8, d = 128, k = 5 698 / 125; and by launches:
+// 8 tokens that fill a cache of 48, 32 units, d = 128 10.3 / 18.5; one of 310, M = 24 18.6 / 105.
 LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B, int c0) {
     const lococo_config& c = h->cfg;
     LoopPlan best{0, 0, 0};

@@ -5,8 +5,8 @@
 // against it, and everything else is latency. What the kernel does about either:
 //  - more units than SMs: two CTAs per SM, one unit each, in half an SM's shared memory and TMEM (decode_shared_kernel): while one
 //    waits for rows, exchanges or stores, the other's MMAs (72 cycles each at N = 144) have the tensor pipe. (One CTA of two units per SM,
-//    a weight tile for both, halves the weights' traffic but puts its latencies one after the other. k = 21: 150 units 27.1 -> 24.8 us,
-//    296 28.9 -> 26.9, 300 51.4 -> 39.2, 512 52.7 -> 47.3, 1536 153 -> 131; k = 5: 150 18.7 -> 16.6, 512 37.0 -> 30.4. Bound now: shared memory,
+//    a weight tile for both, halves the weights' traffic but puts its latencies one after the other. Per step of a graph of 100, k = 21: 150 units 27.1 -> 24.8 us,
+//    296 28.9 -> 26.9, 300 51.4 -> 39.2, 512 52.7 -> 47.3 (a step that is waited for 53.3 -> 50.9), 1536 153 -> 131; k = 5: 150 18.7 -> 16.6, 512 37.0 -> 30.4. Bound now, by count: shared memory,
 //    whose 128 bytes per cycle an MMA's operands and the arriving weights take for about 100 of its cycles);
 //  - few units: a unit is shared by a cluster of 2 or 4 CTAs. Each takes its share of the taps, with its weight tiles
 //    requested before the kernel waits for anything; the partial logits meet through distributed shared memory (a CTA

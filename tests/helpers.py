@@ -1,4 +1,6 @@
 """Shared helpers of the GPU parity tests: upload, error metrics."""
+import ctypes
+
 import numpy as np
 import torch
 
@@ -42,3 +44,17 @@ def assert_close(got: np.ndarray, ref: np.ndarray, dtype: str, what: str = ""):
             f"{what}: max abs {max_abs:.3e} (<= {BF16_MAX_ABS}), mean rel {mean_rel:.3e} (<= {BF16_MEAN_REL})"
     else:
         assert rel <= F32_REL, f"{what}: rel {rel:.3e} (<= {F32_REL})"
+
+
+class _LoopPlan(ctypes.Structure):
+    _fields_ = [("ctas", ctypes.c_int), ("chain_warps", ctypes.c_int), ("tile", ctypes.c_int)]
+
+
+def loop_plan(ctx, L, B, cache_len=0):
+    """How the library runs a small fp32 loop (an internal function of its): CTAs per unit (0: as launches), warps that update the
+    cache, convolution tile (0, 1, 2: 4, 3, 2 slots x 8 positions; 3: 2 x 4)."""
+    from paper_2406_05317_b200 import api
+    plan = api.raw()["_ZN6lococo14simt_loop_planEPK13lococo_handleiii"]
+    plan.argtypes, plan.restype = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int], _LoopPlan
+    p = plan(ctx.handle, L, B, cache_len)
+    return p.ctas, p.chain_warps, p.tile

@@ -26,6 +26,26 @@ def test_grouped_backward(batch, heads, d, M, B, L, k, c_mult, per_head, bias):
     check_backward(w, bias=bias)
 
 
+@pytest.mark.parametrize("batch,heads,d,M,B,L,k,c_mult,groups", [
+    (1, 1, 64, 17, 33, 150, 7, 1, 1),
+    (2, 3, 64, 48, 100, 403, 5, 1, 1),
+    (1, 2, 64, 40, 20, 130, 63, 1, 1),
+    (1, 2, 128, 20, 7, 45, 9, 2, 1),
+    (5, 32, 64, 16, 16, 50, 5, 1, 1),
+    (1, 16, 128, 48, 512, 5632, 3, 1, 0),
+    (1, 8, 128, 48, 512, 10752, 3, 1, 2),
+    (1, 1, 64, 2, 300, 700, 1, 1, 1),
+    (1, 1, 64, 40, 30, 60, 5, 1, 0),                  # a fill step and one compress step: no chain
+])
+def test_which_calls_go_in_groups(batch, heads, d, M, B, L, k, c_mult, groups):
+    # The way that the calls above are there for: five launches per group behind that of delta, or two and four per step.
+    t = Training(wl.Workload("grouped_way", 38, batch=batch, heads=heads, d=d, M=M, B=B, k=k, L=L, dtype="f32", weights_per_head=True, qkv_scale=1.0,
+                             g_std=0.05, c_in_mult=c_mult))
+    launches = t.backward(torch.empty(t.scratch_bytes, dtype=torch.uint8, device="cuda"))[1]
+    compress = [min(M, n * B) + min(B, L - n * B) > M for n in range(-(-L // B))]
+    assert launches == (1 + 5 * groups if groups else 2 + sum(4 if x else 2 for x in compress))
+
+
 class Training:
     """A forward pass with its snapshots; backward passes of it with a scratch of the test's own."""
 

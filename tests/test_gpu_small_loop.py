@@ -1,11 +1,11 @@
-"""fp32 sequences small enough for the single-launch chunk loop (a block per unit): edges of its 4 x 4 tiles, both head
-sizes, stacked input, protected slots, a resumed cache, snapshots for the backward pass. Against the float64 oracle."""
+"""fp32 sequences small enough for the single-launch chunk loop (a cluster of 1 to 16 CTAs per unit): edges of its tiles and clusters, both
+head sizes, stacked input, protected slots, a resumed cache, snapshots for the backward pass. Against the float64 oracle."""
 import numpy as np
 import pytest
 import torch
 
 from paper_2406_05317_b200 import workloads as wl
-from tests.helpers import assert_close, to_device, to_host
+from tests.helpers import assert_close, loop_plan, to_device, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -69,7 +69,7 @@ def test_the_loop_is_timed_on_request():
 
 
 @pytest.mark.parametrize("batch,heads,d,M,B,L,k,c_mult,prot", [
-    (1, 1, 64, 17, 33, 150, 7, 1, 0),         # the widest clusters: CTAs of one and of two slots, of two and of three queries
+    (1, 1, 64, 17, 33, 150, 7, 1, 0),         # wide clusters: CTAs of one and of two slots, of two and of three queries
     (1, 1, 64, 3, 40, 130, 9, 2, 1),          # fewer slots than CTAs would fit
     (3, 4, 64, 30, 21, 104, 5, 1, 5),         # CTAs with and without protected slots
     (2, 20, 128, 13, 9, 48, 3, 1, 0),         # clusters of a few CTAs; fill steps first
@@ -135,3 +135,21 @@ def test_one_chunk_calls_back_to_back():
         return best
 
     assert call_us(2) < 1.25 * call_us(1)
+
+
+@pytest.mark.parametrize("batch,heads,d,M,B,L,k,c_mult,prot,ctas,tile", [
+    (1, 1, 64, 17, 33, 150, 7, 1, 0, range(9, 17), 3),       # (the cases above: what they say they cover)
+    (1, 1, 64, 3, 40, 130, 9, 2, 1, range(2, 4), 2),
+    (3, 4, 64, 30, 21, 104, 5, 1, 5, range(4, 17), 2),
+    (2, 20, 128, 13, 9, 48, 3, 1, 0, range(2, 5), 2),
+    (5, 30, 64, 18, 26, 120, 5, 1, 0, [1], 1),
+    (1, 2, 64, 65, 30, 190, 11, 1, 0, range(9, 17), 2),
+    (1, 1, 64, 16, 90, 363, 3, 1, 3, [16], 2),               # and the widest cluster, a slot each
+    (1, 8, 64, 64, 90, 275, 3, 1, 0, range(8, 17), 0),       # tiles of four slots
+    (5, 15, 64, 15, 45, 183, 3, 2, 2, [1, 2], None),
+])
+def test_small_loop_plans(batch, heads, d, M, B, L, k, c_mult, prot, ctas, tile):
+    from paper_2406_05317_b200 import api
+    plan = loop_plan(api.Lococo(batch, heads, d, M, k, B, dtype=torch.float32, c_in=c_mult * d), L, B)
+    assert plan[0] in ctas and (tile is None or plan[2] == tile), plan
+    test_small_loop_clusters(batch, heads, d, M, B, L, k, c_mult, prot)
