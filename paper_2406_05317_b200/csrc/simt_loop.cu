@@ -429,10 +429,11 @@ ClusterKernel loop_state;      // of the kernel that is asked how many clusters 
 //   here      3 + rounds of clusters x (2.6 for zeros and weights, 2.4 and the work's share per compress step, 1.5 and the attention per fill step)
 //   launches  1.4 + per step the attention's rounds of one block per SM; per fill step 3.6, per compress step the convolution's and the blends' rounds
 // A compress step here is fitted to 44 shapes with every cluster size each, the rest to 260 calls both ways (units 1 to 2000, M and B up to 110
-// and 150, one to twelve chunks, from empty and full caches); of 220 others, 212 go the way that is within 2 % of the faster one, the worst takes
-// twice as long (617 units, M = 54, twelve chunks of 2: 3715 by launches, 1759 here). Launches / this, us per call: 256 tokens of one unit, M = B = 16, d = 64, k = 5
-// 263 / 41; 777 tokens of 8 units, M = 48, B = 100 180 / 72; two chunks of 16 of 1600 units, M = 8, d = 128, k = 5 698 / 125; and by launches:
-// 8 tokens that fill a cache of 48, 32 units, d = 128 10.3 / 18.5; one of 310, M = 24 18.6 / 105.
+// and 150, one to twelve chunks, from empty and full caches). Launches have to be estimated 15 % faster: of 220 other calls 213 went within 3 % of the
+// faster way without that, the worst at twice its time, and 215 with it, the worst at 1.46 times (583 units, M = 8, one chunk of 132: 340 us by
+// launches, 497 here). Launches / this, us per call: 256 tokens of one unit, M = B = 16, d = 64, k = 5 263 / 41; 777 tokens of 8 units, M = 48,
+// B = 100 180 / 72; two chunks of 16 of 1600 units, M = 8, d = 128, k = 5 698 / 125; twelve chunks of 2 of 617 units, M = 54, d = 64, k = 9
+// 3715 / 1759; and by launches: 8 tokens that fill a cache of 48, 32 units, d = 128 10.3 / 18.5; one of 310, M = 24 18.6 / 105.
 LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B, int c0) {
     const lococo_config& c = h->cfg;
     LoopPlan best{0, 0, 0};
@@ -448,7 +449,7 @@ LoopPlan simt_loop_plan(const lococo_handle* h, int L, int B, int c0) {
         const double tiles = (double)(((int)S + PT - 1) / PT) * ((c.M + OT - 1) / OT) * h->units, splits = std::max(1.0, std::min(std::floor(6 * kSMs / tiles), c.c_in / 32.0));
         const double conv = taps * std::max(1 / splits, tiles / (4 * kSMs)), blends = std::floor((S + 63) / 64) * std::max(1.0, (c.M + 15) / 16 * d2 / 64 * h->units / (6 * kSMs));
         auto attention = [&](double n) { return 3.2 * std::max(1.0, (double)h->units * ((B + 31) / 32) / kSMs) * (1 + std::floor(n / 64)) * c.head_dim / 64; };
-        least = 1.4 + fills * (3.6 + attention(fill_keys)) + compresses * (0.094 * conv + 5.6 * blends + attention(S));
+        least = (1.4 + fills * (3.6 + attention(fill_keys)) + compresses * (0.094 * conv + 5.6 * blends + attention(S))) / 0.85;
     }
     const std::atomic<int>* resident = resident_clusters(loop_state, small_loop_kernel<64, 16>, kMaxSmem, kThreads);
     for (int ctas = 1; resident && ctas <= std::min(kMaxCluster, c.M); ctas = next_cluster(ctas)) {
